@@ -49,21 +49,16 @@ __device__ __forceinline__ void batch_warp(const BatchLat &L, const S *fin, S *f
     const int k = (i && nb(bits, OPP(i))) ? OPP(i) * P + self : i * P + src[i];
     h[i] = Store<S>::ld(fin, k, L.inv_scale);
   }
-  const float d = ((h[0] + h[1]) + (h[2] + h[3])) + ((h[4] + h[5]) + (h[6] + h[7])) + h[8];
-  float jx, jy, jxl = 0.f, jyl = 0.f;
-  if (L.pm) {
-    momentum_exact(h, jx, jxl, jy, jyl);
-  } else {
-    jx = (h[1] - h[3]) + (h[5] - h[7]) + (h[8] - h[6]);
-    jy = (h[2] - h[4]) + (h[5] - h[7]) + (h[6] - h[8]);
-  }
-  const float rho = L.rho_ref + d;
-  const float Fx = L.fx + rho * L.ax, Fy = L.fy + rho * L.ay;
-  const float ir = 1.0f / rho;
-  const float mx = jx + (jxl + L.tau * Fx), my = jy + (jyl + L.tau * Fy);
-  const float ux = mx * ir, uy = my * ir;
+  Node1<float> n;
+  if (L.pm) moments1<float, true, false>(h, L.rho_ref, 1.0f, n);
+  else moments1<float, false, false>(h, L.rho_ref, 1.0f, n);
+  n.Fx = vfma(n.rho, L.ax, L.fx);
+  n.Fy = vfma(n.rho, L.ay, L.fy);
+  if (L.pm) shift1<float, true>(L.tau, n);
+  else shift1<float, false>(L.tau, n);
   float heq[9];
-  equilibrium_pairs(d, rho, ux, uy, mx, my, 1.0f / 9.0f, 1.0f / 36.0f, heq);
+  equilibrium1<float, false>(n, 1.0f, 1.0f / 9.0f, 1.0f / 36.0f, heq);
+  relax(h, heq, L.omega, 1.0f - L.omega);
   if (L.sr) {
     // stochastic rounding as in the single-lattice kernels: one hash per
     // node and launch, a linear congruential step per pair of stores
@@ -71,15 +66,15 @@ __device__ __forceinline__ void batch_warp(const BatchLat &L, const S *fin, S *f
 #pragma unroll
     for (int i = 0; i < 8; i += 2) {
       r = r * 1664525u + 1013904223u;
-      Store<S>::st2_dither(fout, i * P + self, (i + 1) * P + self, (h[i] + L.omega * (heq[i] - h[i])) * L.scale,
-                           (h[i + 1] + L.omega * (heq[i + 1] - h[i + 1])) * L.scale, r);
+      Store<S>::st2_dither(fout, i * P + self, (i + 1) * P + self, vmul(h[i], L.scale),
+                           vmul(h[i + 1], L.scale), r);
     }
     r = r * 1664525u + 1013904223u;
-    Store<S>::st_dither(fout, 8 * P + self, (h[8] + L.omega * (heq[8] - h[8])) * L.scale, r);
+    Store<S>::st_dither(fout, 8 * P + self, vmul(h[8], L.scale), r);
   } else {
 #pragma unroll
     for (int i = 0; i < 9; i++)
-      Store<S>::st(fout, i * P + self, h[i] + L.omega * (heq[i] - h[i]), L.scale);
+      Store<S>::st(fout, i * P + self, h[i], L.scale);
   }
 }
 

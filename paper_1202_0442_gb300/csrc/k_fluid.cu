@@ -32,6 +32,8 @@
 // refreshes them around nodes that grow solid): two bytes per node in place
 // of the mask-word arithmetic that otherwise dominated the streaming
 // kernel's instruction count.
+#include <algorithm>
+
 #include "lbcollide.cuh"
 #include "lbpdl.cuh"
 #include "lbsolute.cuh"
@@ -123,14 +125,13 @@ constexpr uint32_t DIAG_BITS = (1u << NBPOS(-1, -1)) | (1u << NBPOS(1, -1)) | (1
 
 constexpr int LOC_BY = 8;
 
-// SR: 0 rounding read from p.sr_seed, 1 nearest, 2 stochastic (16-bit,
-// not ME).  Scaled 16-bit storage without ME runs folded (collide_store).
+// SR: 1 nearest, 2 stochastic (16-bit, not ME).  RX: the form of relax.  Scaled 16-bit storage without ME runs folded (collide_store).
 // The update of node (x, y) given its neighbour code (called by every lane
 // of a warp: the warp votes on its solid lanes).  Returns false on solid
 // nodes and row padding.  uo, if given, receives the node's solvent
 // velocity of Eq. (4).  SLIP: the slip/mixed/hybrid boundary styles (a
 // compile-time switch: the noslip kernels carry none of its registers).
-template <class S, int NC, bool ME, bool PM, int SR, bool SLIP>
+template <class S, int NC, bool ME, bool PM, int SR, bool SLIP, int RX = 0>
 __device__ __forceinline__ bool fluid_node(const FluidArgs &p, int x, int y, uint32_t bits,
                                            float *uo = nullptr) {
   constexpr bool FOLD = Store<S>::kScaled && !ME;
@@ -167,14 +168,18 @@ __device__ __forceinline__ bool fluid_node(const FluidArgs &p, int x, int y, uin
       slip_fix<S>(p, c, (const S *)p.fin + (size_t)c * 9 * g.plane, x, y, bits, linv, h[c]);
   }
   if (p.nopen) apply_openings<NC>(p, x, y, h, FOLD ? p.scale : 1.0f);
-  float F[NC][2];
+  if constexpr (ME) {
+    float F[NC][2];
 #pragma unroll
-  for (int c = 0; c < NC; c++) F[c][0] = F[c][1] = 0.f;
-  collide_store<S, NC, ME, PM, FOLD, SR>(p, x, y, bits, h, F, uo);
+    for (int c = 0; c < NC; c++) F[c][0] = F[c][1] = 0.f;
+    collide_store_me<S, NC>(p, x, y, bits, h, F);
+  } else {
+    collide_store<S, PM, FOLD, SR, RX>(p, x, y, bits, h[0], uo);
+  }
   return true;
 }
 
-template <class S, int NC, bool ME, bool PM, int SR, bool SLIP>
+template <class S, int NC, bool ME, bool PM, int SR, bool SLIP, int RX>
 __global__ void __launch_bounds__(32 * LOC_BY, ((NC == 1 && !ME && !PM) ? (SLIP ? 6 : 8) : 4) * 8 / LOC_BY)
     k_fluid_local(const FluidArgs p) {
   dep_wait();
@@ -182,7 +187,7 @@ __global__ void __launch_bounds__(32 * LOC_BY, ((NC == 1 && !ME && !PM) ? (SLIP 
   const int y = p.g.clo + blockIdx.y * LOC_BY + threadIdx.y;
   if (y >= p.g.chi) return;
   // x < pitch: the grid covers whole 32-node words
-  fluid_node<S, NC, ME, PM, SR, SLIP>(p, x, y, __ldg(p.nbc + (size_t)y * p.g.pitch + x));
+  fluid_node<S, NC, ME, PM, SR, SLIP, RX>(p, x, y, __ldg(p.nbc + (size_t)y * p.g.pitch + x));
 }
 
 // One fluid and one solute iteration of a single-component lattice in one
@@ -301,7 +306,7 @@ __global__ void __launch_bounds__(SC_TX *SC_TY, 4) k_fluid_sc(const FluidArgs p)
     F[c][0] = -p.G * self * sx;
     F[c][1] = -p.G * self * sy;
   }
-  collide_store<S, NC, true>(p, x, y, bits, h, F);
+  collide_store_me<S, NC>(p, x, y, bits, h, F);
 }
 
 template <class S>
@@ -363,8 +368,10 @@ __global__ void k_nbcode(const uint32_t *mask, uint16_t *nbc, const Geometry g, 
 template <class S, int NC, bool ME, bool PM, int SR>
 void launch_local(const FluidArgs &a, cudaStream_t s) {
   dim3 blk(32, LOC_BY), grd((a.g.nx + 31) / 32, (a.g.chi - a.g.clo + LOC_BY - 1) / LOC_BY);
-  if (a.slip) launch_pdl(k_fluid_local<S, NC, ME, PM, SR, true>, grd, blk, 0, s, a);
-  else launch_pdl(k_fluid_local<S, NC, ME, PM, SR, false>, grd, blk, 0, s, a);
+  if (a.slip) launch_pdl(k_fluid_local<S, NC, ME, PM, SR, true, 0>, grd, blk, 0, s, a);
+  else if constexpr (ME || PM) launch_pdl(k_fluid_local<S, NC, ME, PM, SR, false, 0>, grd, blk, 0, s, a);
+  else if (a.omega[0] >= 1.0f) launch_pdl(k_fluid_local<S, NC, ME, PM, SR, false, 1>, grd, blk, 0, s, a);
+  else launch_pdl(k_fluid_local<S, NC, ME, PM, SR, false, 2>, grd, blk, 0, s, a);
 }
 
 template <class S>
@@ -383,12 +390,10 @@ int launch_fluid_t(int nc, bool sc, bool me, const FluidArgs &a, cudaStream_t s)
     }
   } else {
     if (nc == 1) {
-      if (me) {
-        if (a.pm) launch_local<S, 1, true, true, 0>(a, s);
-        else launch_local<S, 1, true, false, 0>(a, s);
-      } else if (a.sr_seed) {
-        if (a.pm) launch_local<S, 1, false, true, 2>(a, s);
-        else launch_local<S, 1, false, false, 2>(a, s);
+      if (sizeof(S) == 2 && a.sr_seed) {
+        constexpr int SR = sizeof(S) == 2 ? 2 : 1;
+        if (a.pm) launch_local<S, 1, false, true, SR>(a, s);
+        else launch_local<S, 1, false, false, SR>(a, s);
       } else {
         if (a.pm) launch_local<S, 1, false, true, 1>(a, s);
         else launch_local<S, 1, false, false, 1>(a, s);
@@ -431,6 +436,45 @@ int launch_fluid_solute(int storage, int q, const FluidArgs &a, const SoluteArgs
       return a.sr_seed ? launch_fluid_solute_t<__nv_bfloat16, 2>(q, a, sa, s)
                        : launch_fluid_solute_t<__nv_bfloat16, 1>(q, a, sa, s);
     default: return launch_fluid_solute_t<float, 1>(q, a, sa, s);
+  }
+}
+
+int launch_march_f32(const MarchArgs &a, dim3 grid, dim3 block, cudaStream_t s);
+int launch_march_f16(const MarchArgs &a, dim3 grid, dim3 block, cudaStream_t s);
+int launch_march_bf16(const MarchArgs &a, dim3 grid, dim3 block, cudaStream_t s);
+
+int launch_march(int storage, MarchArgs &a, int sms, cudaStream_t s) {
+  const Geometry &g = a.f.g;
+  // strips of equal width
+  const int n = (g.nx + MARCH_COLS - 1) / MARCH_COLS;
+  a.sw = ((g.nx + n - 1) / n + 1) & ~1;
+  const int all = (g.nx + a.sw - 1) / a.sw;
+  const bool edges = a.f.nopen > 0;
+  a.last = (all - 1) * a.sw;
+  a.x0 = edges ? a.sw : 0;
+  a.strips = edges ? std::max(all - 2, 0) : all;
+  // warps of a block: the number of adjacent strips that wastes the fewest
+  int wpb = 4;
+  while (wpb > 1 && (a.strips + wpb - 1) / wpb * wpb > (a.strips + wpb - 2) / (wpb - 1) * (wpb - 1)) wpb--;
+  if (!a.strips) wpb = 2;
+  a.bx = (a.strips + wpb - 1) / wpb;
+  // Rows per warp: the fewest with which every block is resident at once
+  // (16 warps of 128 registers per SM; shorter segments in more than one
+  // wave repeat more rows at their ends: porous 1024^2 FP32 7.8 us per
+  // iteration with one wave, 8.5 with one and a half or two).  The border
+  // strips take half as many (FP16 2003 x 1501: 23.2 us per iteration with
+  // as many rows, 21.1 with half, 21.8 with a third).
+  const int slots = sms * (16 / wpb);
+  for (a.seg = 2;; a.seg++) {
+    a.eseg = (a.seg + 1) / 2;
+    a.eb = edges ? (2 * ((g.ny + a.eseg - 1) / a.eseg) + wpb - 1) / wpb : 0;
+    if (a.seg >= g.ny || a.eb + a.bx * ((g.ny + a.seg - 1) / a.seg) <= slots) break;
+  }
+  const dim3 grid(a.eb + a.bx * ((g.ny + a.seg - 1) / a.seg)), block(32, wpb);
+  switch (storage) {
+    case ST_FP16: return launch_march_f16(a, grid, block, s);
+    case ST_BF16: return launch_march_bf16(a, grid, block, s);
+    default: return launch_march_f32(a, grid, block, s);
   }
 }
 

@@ -1,0 +1,10 @@
+// k_march_bf16.cu -- k_march compiled for __nv_bfloat16 storage.
+#include "k_march.cuh"
+
+namespace lbk {
+
+int launch_march_bf16(const MarchArgs &a, dim3 grid, dim3 block, cudaStream_t s) {
+  return a.f.sr_seed ? launch_march_t<__nv_bfloat16, 2>(a, grid, block, s) : launch_march_t<__nv_bfloat16, 1>(a, grid, block, s);
+}
+
+}  // namespace lbk

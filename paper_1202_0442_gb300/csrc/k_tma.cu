@@ -245,8 +245,7 @@ __global__ void __launch_bounds__(TT_THREADS, 3) k_fluid_tma(const FluidArgs p, 
         h[0][i] = Store<S>::ld_smem(sb, off, linv);
       }
       if (p.nopen) apply_openings<1>(p, x, y, h, FOLD ? p.scale : 1.0f);
-      const float F[1][2] = {{0.f, 0.f}};
-      collide_store<S, 1, false, false, FOLD, SR>(p, x, y, bits, h, F);
+      collide_store<S, false, FOLD, SR>(p, x, y, bits, h[0]);
     }
     if (kn < ntiles && tid < L::ROWS * L::MW) msk0[(s ^ 1) * L::ROWS * L::MW + tid] = mnext;
     __syncthreads();

@@ -5,7 +5,7 @@
 // populations come from.
 #pragma once
 
-#include "lbdev.cuh"
+#include "lbarith.cuh"
 
 namespace lbk {
 
@@ -17,41 +17,15 @@ __device__ __forceinline__ uint32_t rnd(uint32_t seed, int self, int c, int i) {
                (0x85ebca6bu * (uint32_t)(i + 1)));
 }
 
-// momentum sum_i e_i f_i of one component as an unevaluated sum hi + lo,
-// every addition error-free (two_sum): a moment rounded to FP32 feeds its
-// rounding error back into the state as a spurious force (the collision
-// relaxes toward the computed momentum), which in slow force-driven flows
-// is comparable with the force itself
-__device__ __forceinline__ void momentum_exact(const float (&f)[9], float &jx, float &jxl, float &jy,
-                                               float &jyl) {
-  float a, ea, b, eb, d, ed, s, es, t, et;
-  two_sum(f[1], -f[3], a, ea);
-  two_sum(f[5], -f[7], b, eb);
-  two_sum(f[8], -f[6], d, ed);
-  two_sum(a, b, s, es);
-  two_sum(s, d, t, et);
-  jx = t;
-  jxl = ((ea + eb) + (ed + es)) + et;
-  two_sum(f[2], -f[4], a, ea);
-  two_sum(f[5], -f[7], b, eb);
-  two_sum(f[6], -f[8], d, ed);
-  two_sum(a, b, s, es);
-  two_sum(s, d, t, et);
-  jy = t;
-  jyl = ((ea + eb) + (ed + es)) + et;
-}
-
-// moments, forces, equilibrium velocity, BGK and the stores of one node.
-// Fsc: interforce already evaluated (zero when off).  ME: mass-exact
-// collision (see below).  PM: the momentum as an exact hi + lo sum (single
-// component; the storage flag LB_PRECISE_MOMENTUM).  FOLD (scaled 16-bit
-// storage, not ME): h arrives and leaves in the stored units 2^s h, so the
-// loads and stores skip their scale factors; the moments are unscaled once
-// and the equilibrium is formed directly in stored units.  SR: 0 read
-// p.sr_seed, 1 round to nearest, 2 stochastic rounding.
-template <class S, int NC, bool ME, bool PM = false, bool FOLD = false, int SR = 0>
-__device__ __forceinline__ void collide_store(const FluidArgs &p, int x, int y, uint32_t bits,
-                                              float (&h)[NC][9], const float (&Fsc)[NC][2],
+// moments, forces, equilibrium velocity, BGK and the stores of one node of a
+// single-component lattice.  PM: the momentum as an exact hi + lo sum (the
+// storage flag LB_PRECISE_MOMENTUM).  FOLD (scaled 16-bit storage): h
+// arrives and leaves in the stored units 2^s h, so the loads and stores skip
+// their scale factors; the moments are unscaled once and the equilibrium is
+// formed directly in stored units.  SR: 1 round to nearest, 2 stochastic
+// rounding.
+template <class S, bool PM, bool FOLD, int SR, int RX = 0>
+__device__ __forceinline__ void collide_store(const FluidArgs &p, int x, int y, uint32_t bits, float (&h)[9],
                                               float *uo = nullptr) {
   const Geometry &g = p.g;
   const int self = y * g.pitch + x;
@@ -59,25 +33,111 @@ __device__ __forceinline__ void collide_store(const FluidArgs &p, int x, int y, 
   // whether the lattice is held whole or in slabs
   const int hself = self + g.yoff * g.pitch;
   const int P = (int)g.plane;
-  float drho[NC], rho[NC], jx[NC], jy[NC], jxl[NC], jyl[NC], Fx[NC], Fy[NC];
+  Node1<float> n;
   // stored units -> physical units (a power of two: exact)
   const float un = FOLD ? p.inv_scale : 1.0f;
+  moments1<float, PM, FOLD>(h, p.rho_ref[0], un, n);
+  n.Fx = vfma(n.rho, p.ax[0], p.fx[0]);
+  n.Fy = vfma(n.rho, p.ay[0], p.fy[0]);
+  if (p.ads[0]) {
+    float sx, sy;
+    wall_sum(bits, sx, sy);
+    const float psi = p.ads_psi0[0] * expf(-p.ads_rho0[0] / n.rho);
+    n.Fx -= p.Gads[0] * psi * sx;
+    n.Fy -= p.Gads[0] * psi * sy;
+  }
+  shift1<float, PM>(p.tau[0], n);
+  S *out = (S *)p.fout;
+  float heq[9];
+  equilibrium1<float, FOLD>(n, p.scale, p.wa[0], p.wd[0], heq);
+  relax<RX>(h, heq, p.omega[0], p.keep);
+  const float sc = FOLD ? 1.0f : p.scale;
+  if (SR == 2) {
+    // stochastic rounding: one hash per node, then a linear congruential
+    // sequence, one step per pair of stores (each state is uniform for a
+    // uniformly random start, so both dithers of the paired conversion are
+    // uniform: unbiased rounding); the ninth store takes the single
+    // conversion's high bits
+    uint32_t r = rnd(p.sr_seed, hself, 0, 0);
+#pragma unroll
+    for (int i = 0; i < 8; i += 2) {
+      r = r * 1664525u + 1013904223u;
+      Store<S>::st2_dither(out, i * P + self, (i + 1) * P + self, vmul(h[i], sc), vmul(h[i + 1], sc), r);
+    }
+    r = r * 1664525u + 1013904223u;
+    Store<S>::st_dither(out, 8 * P + self, vmul(h[8], sc), r);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 9; i++) Store<S>::st(out, i * P + self, h[i], sc);
+  }
+  const float px = vadd(n.jx, vfma(0.5f, n.Fx, n.jxl)), py = vadd(n.jy, vfma(0.5f, n.Fy, n.jyl));
+  if (p.fields) {
+    p.fields[self] = n.drho;
+    p.fields[P + self] = px;
+    p.fields[2 * P + self] = py;
+    p.fields[3 * P + self] = equilibrium_sum(heq, un);
+  }
+  if (p.uout || uo) {
+    // the solvent velocity of Eq. (4)
+    const float vx = px / n.rho, vy = py / n.rho;
+    if (uo) {
+      uo[0] = vx;
+      uo[1] = vy;
+    }
+    if (p.uout) {
+      p.uout[self] = vx;
+      p.uout[P + self] = vy;
+    }
+  }
+}
+
+// the equilibrium of lbarith.cuh for the mass-exact collision, in plain
+// expressions
+__device__ __forceinline__ void equilibrium_pairs(float drho, float rho, float ux, float uy,
+                                                  float mx, float my, float wa, float wd,
+                                                  float (&heq)[9]) {
+  const float q = rho * (ux * ux + uy * uy);
+  const float sp = ux + uy, sm = uy - ux;  // e5.u and e6.u
+  const float d9 = drho * wa, d36 = drho * wd;
+  const float A1 = d9 + 0.5f * rho * ux * ux - q * (1.0f / 6.0f);
+  const float A2 = d9 + 0.5f * rho * uy * uy - q * (1.0f / 6.0f);
+  const float A5 = d36 + 0.125f * rho * sp * sp - q * (1.0f / 24.0f);
+  const float A6 = d36 + 0.125f * rho * sm * sm - q * (1.0f / 24.0f);
+  const float B5 = rho * sp * (1.0f / 12.0f);
+  const float B6 = rho * sm * (1.0f / 12.0f);
+  const float B1 = 0.5f * mx - B5 + B6;
+  const float B2 = 0.5f * my - B5 - B6;
+  heq[1] = A1 + B1;
+  heq[3] = A1 - B1;
+  heq[2] = A2 + B2;
+  heq[4] = A2 - B2;
+  heq[5] = A5 + B5;
+  heq[7] = A5 - B5;
+  heq[6] = A6 + B6;
+  heq[8] = A6 - B6;
+  heq[0] = drho - 2.0f * ((A1 + A2) + (A5 + A6));
+}
+
+// the same node update with the mass-exact collision (see below): two
+// components, or interforce.  Fsc: interforce already evaluated (zero when
+// off).
+template <class S, int NC>
+__device__ __forceinline__ void collide_store_me(const FluidArgs &p, int x, int y, uint32_t bits,
+                                                 float (&h)[NC][9], const float (&Fsc)[NC][2]) {
+  const Geometry &g = p.g;
+  const int self = y * g.pitch + x;
+  // the node's slot in the whole lattice: the random words are the same
+  // whether the lattice is held whole or in slabs
+  const int hself = self + g.yoff * g.pitch;
+  const int P = (int)g.plane;
+  float drho[NC], rho[NC], jx[NC], jy[NC], Fx[NC], Fy[NC];
 #pragma unroll
   for (int c = 0; c < NC; c++) {
     const float(&f)[9] = h[c];
-    drho[c] = (((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8]) * un;
+    drho[c] = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
     rho[c] = p.rho_ref[c] + drho[c];
-    if (PM && NC == 1) {
-      momentum_exact(f, jx[c], jxl[c], jy[c], jyl[c]);
-    } else {
-      jx[c] = (f[1] - f[3]) + (f[5] - f[7]) + (f[8] - f[6]);
-      jy[c] = (f[2] - f[4]) + (f[5] - f[7]) + (f[6] - f[8]);
-      jxl[c] = jyl[c] = 0.f;
-    }
-    jx[c] *= un;
-    jy[c] *= un;
-    jxl[c] *= un;
-    jyl[c] *= un;
+    jx[c] = (f[1] - f[3]) + (f[5] - f[7]) + (f[8] - f[6]);
+    jy[c] = (f[2] - f[4]) + (f[5] - f[7]) + (f[6] - f[8]);
     Fx[c] = p.fx[c] + rho[c] * p.ax[c] + Fsc[c][0];
     Fy[c] = p.fy[c] + rho[c] * p.ay[c] + Fsc[c][1];
     if (p.ads[c]) {
@@ -92,8 +152,8 @@ __device__ __forceinline__ void collide_store(const FluidArgs &p, int x, int y, 
   // carries, the latter formed without a division
   float uex[NC], uey[NC], mxt[NC], myt[NC];
   if (NC == 1) {
-    mxt[0] = PM ? jx[0] + (jxl[0] + p.tau[0] * Fx[0]) : jx[0] + p.tau[0] * Fx[0];
-    myt[0] = PM ? jy[0] + (jyl[0] + p.tau[0] * Fy[0]) : jy[0] + p.tau[0] * Fy[0];
+    mxt[0] = jx[0] + p.tau[0] * Fx[0];
+    myt[0] = jy[0] + p.tau[0] * Fy[0];
     const float ir = 1.0f / rho[0];
     uex[0] = mxt[0] * ir;
     uey[0] = myt[0] * ir;
@@ -119,124 +179,158 @@ __device__ __forceinline__ void collide_store(const FluidArgs &p, int x, int y, 
   for (int c = 0; c < NC; c++) {
     S *out = (S *)p.fout + (size_t)c * 9 * P;
     float heq[9];
-    if (FOLD) {
-      // the equilibrium is linear in (drho, rho, rho u): in stored units
-      // it takes 2^s drho, 2^s rho and 2^s rho u at the same velocity
-      const float sc = p.scale;
-      equilibrium_pairs(drho[c] * sc, rho[c] * sc, uex[c], uey[c], mxt[c] * sc, myt[c] * sc, p.wa[c],
-                        p.wd[c], heq);
-    } else {
-      equilibrium_pairs(drho[c], rho[c], uex[c], uey[c], mxt[c], myt[c], p.wa[c], p.wd[c], heq);
-    }
+    equilibrium_pairs(drho[c], rho[c], uex[c], uey[c], mxt[c], myt[c], p.wa[c], p.wd[c], heq);
     const float om = p.omega[c];
-    if (!ME && SR == 2) {
-      // stochastic rounding: one hash per node and component, then a
-      // linear congruential sequence, one step per pair of stores (each
-      // state is uniform for a uniformly random start, so both dithers of
-      // the paired conversion are uniform: unbiased rounding); the ninth
-      // store takes the single conversion's high bits
-      uint32_t r = rnd(p.sr_seed, hself, c, 0);
-      const float sc = FOLD ? 1.0f : p.scale;
+    // Mass-exact collision: when |h| is large (two components, or one far
+    // from rho_ref) the rounding of nine stored values of a slowly
+    // changing state repeats every step and drifts the mass.  Here the
+    // exact sum D of the pulled values and the exact sum S of the eight
+    // stored moving populations are formed with error-free sums, and the
+    // rest population is set to D - S -- the BGK value in exact
+    // arithmetic -- rounded stochastically, so the node's mass is kept
+    // up to an unbiased last-bit step.
+    float Dh = h[c][0], Dl = 0.f;
 #pragma unroll
-      for (int i = 0; i < 8; i += 2) {
-        const float v0 = (h[c][i] + om * (heq[i] - h[c][i])) * sc;
-        const float v1 = (h[c][i + 1] + om * (heq[i + 1] - h[c][i + 1])) * sc;
-        r = r * 1664525u + 1013904223u;
-        Store<S>::st2_dither(out, i * P + self, (i + 1) * P + self, v0, v1, r);
-      }
-      r = r * 1664525u + 1013904223u;
-      Store<S>::st_dither(out, 8 * P + self, (h[c][8] + om * (heq[8] - h[c][8])) * sc, r);
-    } else if (!ME && SR == 1) {
-#pragma unroll
-      for (int i = 0; i < 9; i++)
-        Store<S>::st(out, i * P + self, h[c][i] + om * (heq[i] - h[c][i]), FOLD ? 1.0f : p.scale);
-    } else if (!ME) {
-      uint32_t r = p.sr_seed ? rnd(p.sr_seed, hself, c, 0) : 0u;
-#pragma unroll
-      for (int i = 0; i < 9; i++) {
-        // dither of the 16-bit stores: one hash per node and component,
-        // then a linear congruential sequence (its high bits) per direction
-        r = r * 1664525u + 1013904223u;
-        Store<S>::st(out, i * P + self, h[c][i] + om * (heq[i] - h[c][i]), p.scale,
-                     p.sr_seed ? (r >> 13) | 1u : 0u);
-      }
-    } else {
-      // Mass-exact collision: when |h| is large (two components, or one far
-      // from rho_ref) the rounding of nine stored values of a slowly
-      // changing state repeats every step and drifts the mass.  Here the
-      // exact sum D of the pulled values and the exact sum S of the eight
-      // stored moving populations are formed with error-free sums, and the
-      // rest population is set to D - S -- the BGK value in exact
-      // arithmetic -- rounded stochastically, so the node's mass is kept
-      // up to an unbiased last-bit step.
-      float Dh = h[c][0], Dl = 0.f;
-#pragma unroll
-      for (int i = 1; i < 9; i++) {
-        float s, e;
-        two_sum(Dh, h[c][i], s, e);
-        Dh = s;
-        Dl += e;
-      }
-      float Sh = 0.f, Sl = 0.f;
-#pragma unroll
-      for (int i = 1; i < 9; i++) {
-        // 16-bit dither: an independent hash per store (a linear
-        // congruential sequence per node, as in the plain collision, was
-        // measurably worse for the two-component runs)
-        const uint32_t r = p.sr_seed ? (rnd(p.sr_seed, hself, c, i) | 1u) : 0u;
-        const float v = Store<S>::st_ret(out, i * P + self, h[c][i] + om * (heq[i] - h[c][i]),
-                                         p.scale, p.inv_scale, r);
-        float s, e;
-        two_sum(Sh, v, s, e);
-        Sh = s;
-        Sl += e;
-      }
-      float rh, rl;
-      two_sum(Dh, -Sh, rh, rl);
-      rl += Dl - Sl;
-      float h0, rem;
-      two_sum(rh, rl, h0, rem);
-      if (rem != 0.f && h0 != 0.f) {
-        const int step = ((rem > 0.f) == (h0 > 0.f)) ? 1 : -1;
-        const float nxt = __int_as_float(__float_as_int(h0) + step);
-        // |nxt - h0| is a power of two, so the quotient is exact up to the
-        // fast division's last bit: a probability, compared with a uniform
-        // variate
-        const float pr = __fdividef(fabsf(rem), fabsf(nxt - h0));
-        const float u01 = (float)(rnd(p.step_seed, hself, c, 9) >> 8) * (1.0f / 16777216.0f);
-        if (u01 < pr) h0 = nxt;
-      }
-      const uint32_t r0 = p.sr_seed ? (rnd(p.sr_seed, hself, c, 0) | 1u) : 0u;
-      Store<S>::st(out, self, h0, p.scale, r0);
+    for (int i = 1; i < 9; i++) {
+      float s, e;
+      two_sum(Dh, h[c][i], s, e);
+      Dh = s;
+      Dl += e;
     }
+    float Sh = 0.f, Sl = 0.f;
+#pragma unroll
+    for (int i = 1; i < 9; i++) {
+      // 16-bit dither: an independent hash per store (a linear
+      // congruential sequence per node, as in the plain collision, was
+      // measurably worse for the two-component runs)
+      const uint32_t r = p.sr_seed ? (rnd(p.sr_seed, hself, c, i) | 1u) : 0u;
+      const float v = Store<S>::st_ret(out, i * P + self, h[c][i] + om * (heq[i] - h[c][i]),
+                                       p.scale, p.inv_scale, r);
+      float s, e;
+      two_sum(Sh, v, s, e);
+      Sh = s;
+      Sl += e;
+    }
+    float rh, rl;
+    two_sum(Dh, -Sh, rh, rl);
+    rl += Dl - Sl;
+    float h0, rem;
+    two_sum(rh, rl, h0, rem);
+    if (rem != 0.f && h0 != 0.f) {
+      const int step = ((rem > 0.f) == (h0 > 0.f)) ? 1 : -1;
+      const float nxt = __int_as_float(__float_as_int(h0) + step);
+      // |nxt - h0| is a power of two, so the quotient is exact up to the
+      // fast division's last bit: a probability, compared with a uniform
+      // variate
+      const float pr = __fdividef(fabsf(rem), fabsf(nxt - h0));
+      const float u01 = (float)(rnd(p.step_seed, hself, c, 9) >> 8) * (1.0f / 16777216.0f);
+      if (u01 < pr) h0 = nxt;
+    }
+    const uint32_t r0 = p.sr_seed ? (rnd(p.sr_seed, hself, c, 0) | 1u) : 0u;
+    Store<S>::st(out, self, h0, p.scale, r0);
     if (p.fields) {
       float *fl = p.fields + (size_t)c * NFIELD * P;
       fl[self] = drho[c];
-      fl[P + self] = jx[c] + (jxl[c] + 0.5f * Fx[c]);
-      fl[2 * P + self] = jy[c] + (jyl[c] + 0.5f * Fy[c]);
+      fl[P + self] = jx[c] + 0.5f * Fx[c];
+      fl[2 * P + self] = jy[c] + 0.5f * Fy[c];
       // sum of the equilibrium populations (Mass_eq of the thermo command)
       fl[3 * P + self] = (heq[0] + ((heq[1] + heq[3]) + (heq[2] + heq[4])) +
-                          ((heq[5] + heq[7]) + (heq[6] + heq[8]))) * un;
+                          ((heq[5] + heq[7]) + (heq[6] + heq[8])));
     }
   }
-  if (p.uout || uo) {
+  if (p.uout) {
     // the solvent velocity of Eq. (4)
     float pxs = 0.f, pys = 0.f, rs = 0.f;
 #pragma unroll
     for (int c = 0; c < NC; c++) {
-      pxs += jx[c] + (jxl[c] + 0.5f * Fx[c]);
-      pys += jy[c] + (jyl[c] + 0.5f * Fy[c]);
+      pxs += jx[c] + 0.5f * Fx[c];
+      pys += jy[c] + 0.5f * Fy[c];
       rs += rho[c];
     }
-    const float vx = pxs / rs, vy = pys / rs;
-    if (uo) {
-      uo[0] = vx;
-      uo[1] = vy;
-    }
-    if (p.uout) {
-      p.uout[self] = vx;
-      p.uout[P + self] = vy;
-    }
+    p.uout[self] = pxs / rs;
+    p.uout[P + self] = pys / rs;
+  }
+}
+
+// ---------------------------------------------------------------------
+// inlet/outlet rules in one rotated form.
+//
+// Every wall is mapped onto a canonical one whose inward normal n is e1 and
+// tangent t is e2; canonical slot k then holds direction PERM[wall][k]:
+//   k: 0  1=n  2=t  3=-n  4=-t  5=n+t  6=-n+t  7=-n-t  8=n-t
+// With u_n the velocity along n, S = h0 + h2 + h4 + 2 (h3 + h6 + h7) and
+// a = rho u_n:
+//   velocity styles:  rho = (rho_ref + S)/(1 - u_n), so
+//                     a = (rho_ref + S) u_n/(1 - u_n)
+//   dirichlet:        u_n = (rho - rho_ref - S)/rho, so a = rho - rho_ref - S
+//   h1 = h3 + 2/3 a
+//   h5 = h7 - (h2 - h4)/2 + a/6
+//   h8 = h6 + (h2 - h4)/2 + a/6
+// which is the set of printed rules for each wall and style (inlet: u_n =
+// +v, outlet: u_n = -v), written for deviations h = f - w rho_ref.  Either
+// way a = m S + b with m and b fixed by the opening (and, for a Poiseuille
+// profile, the node's place along it).
+// ---------------------------------------------------------------------
+template <int WALL> __device__ __forceinline__ constexpr int PERM(int k) {
+  // xlo: n=+x t=+y; xhi: n=-x t=+y; ylo: n=+y t=+x; yhi: n=-y t=-x
+  return WALL == 0 ? k
+       : WALL == 1 ? (k == 1 ? 3 : k == 3 ? 1 : k == 5 ? 6 : k == 6 ? 5 : k == 7 ? 8 : k == 8 ? 7 : k)
+       : WALL == 2 ? (k == 1 ? 2 : k == 2 ? 1 : k == 3 ? 4 : k == 4 ? 3 : k == 6 ? 8 : k == 8 ? 6 : k)
+                   : (k == 1 ? 4 : k == 2 ? 3 : k == 3 ? 2 : k == 4 ? 1 : k == 5 ? 7 : k == 7 ? 5 : k);
+}
+
+template <int WALL, class V>
+__device__ __forceinline__ void zou_he(const V (&h)[9], V m, V b, V &h1, V &h5, V &h8) {
+  constexpr int c0 = PERM<WALL>(0), c2 = PERM<WALL>(2), c3 = PERM<WALL>(3), c4 = PERM<WALL>(4), c6 = PERM<WALL>(6),
+                c7 = PERM<WALL>(7);
+  const V S = vfma(vset<V>(2.0f), vadd(vadd(h[c3], h[c6]), h[c7]), vadd(vadd(h[c0], h[c2]), h[c4]));
+  const V a = vfma(S, m, b), d = vsub(h[c2], h[c4]), sixth = vset<V>(1.0f / 6.0f);
+  h1 = vfma(vset<V>(2.0f / 3.0f), a, h[c3]);
+  h5 = vfma(sixth, a, vfma(vset<V>(-0.5f), d, h[c7]));
+  h8 = vfma(sixth, a, vfma(vset<V>(0.5f), d, h[c6]));
+}
+
+template <int WALL>
+__device__ __forceinline__ void zou_he_node(float (&h)[9], float m, float b) {
+  float h1, h5, h8;
+  zou_he<WALL>(h, m, b, h1, h5, h8);
+  h[PERM<WALL>(1)] = h1;
+  h[PERM<WALL>(5)] = h5;
+  h[PERM<WALL>(8)] = h8;
+}
+
+// m and b of component c's rule at coordinate coord along the wall; false
+// if the component has no velocity or density style there.  sc: the units
+// of h (the rule is homogeneous of degree one in h, drho and rho_ref, so
+// scaled storage units take sc = 2^s)
+__device__ __forceinline__ bool opening_mb(const OpenSpan &s, const OpenRule &r, int c, int coord, float rho_ref,
+                                           float sc, float &m, float &b) {
+  const int st = (r.bits >> (3 * c)) & 7;
+  if (st == OPEN_DIRICHLET) {
+    m = -1.0f;
+    b = vmul(r.val[c], sc);
+    return true;
+  }
+  if (st != OPEN_POISEUILLE && st != OPEN_UNIFORM) return false;
+  const float v = (st == OPEN_UNIFORM) ? r.val[c] : poiseuille(r.val[c], s.wa0 >> 2, s.a1, coord);
+  const float un = ((r.bits >> 6) & 1) == 0 ? v : -v;
+  m = __fdiv_rn(un, vsub(1.0f, un));
+  b = vmul(vmul(rho_ref, sc), m);
+  return true;
+}
+
+// apply the velocity/dirichlet rule r of the opening at s to component c's
+// h (in units sc)
+__device__ __forceinline__ void apply_opening(const OpenSpan &s, const OpenRule &r, int c, float (&h)[9],
+                                              int x, int y, float rho_ref, float sc = 1.0f) {
+  const int wall = span_wall(s);
+  float m, b;
+  if (!opening_mb(s, r, c, wall <= 1 ? y : x, rho_ref, sc, m, b)) return;
+  switch (wall) {
+    case 0: zou_he_node<0>(h, m, b); break;
+    case 1: zou_he_node<1>(h, m, b); break;
+    case 2: zou_he_node<2>(h, m, b); break;
+    default: zou_he_node<3>(h, m, b); break;
   }
 }
 

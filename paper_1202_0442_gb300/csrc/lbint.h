@@ -86,6 +86,7 @@ struct FluidArgs {
   float rho_ref[2];
   float scale, inv_scale; // storage scale 2^s and 2^-s (FP16), else 1
   float tau[2], omega[2];
+  float keep;             // 1 - omega[0] (single component)
   float wa[2], wd[2];     // rest-state shares s_1..4, s_5..8 (fluids alpha)
   float fx[2], fy[2];     // aveforce
   float ax[2], ay[2];     // aveacceleration
@@ -108,6 +109,19 @@ struct FluidArgs {
   float slipR[2];
   const float *Rmap;
   int edge_x, edge_y;
+};
+
+// two iterations of a whole single-component lattice in one pass
+// (k_march.cuh): f.sr_seed dithers the first, sr_seed2 the second
+constexpr int MARCH_COLS = 60;
+struct MarchArgs {
+  FluidArgs f;
+  uint32_t sr_seed2;
+  int sw;                  // columns a warp advances (even, <= MARCH_COLS)
+  int x0, strips, seg, bx; // the strips without an opening: first column,
+                           // their number, rows per warp, blocks per row
+  int eb, last, eseg;      // the border strips: blocks (0 without openings),
+                           // first column of the last one, rows per warp
 };
 
 // gradient openings (after collision)
@@ -216,6 +230,7 @@ struct CopyRuns {
 
 // launchers (return the kernel count launched, or -1 on a launch error)
 int launch_fluid(int storage, int nc, bool sc, bool mass_exact, const FluidArgs &a, cudaStream_t s);
+int launch_march(int storage, MarchArgs &a, int sms, cudaStream_t s);
 int launch_gradient(int storage, const GradArgs &a, cudaStream_t s);
 // fluid and solute iteration in one kernel (one component, no interforce,
 // no intersolute, no exact momentum pairs, streaming kernel)

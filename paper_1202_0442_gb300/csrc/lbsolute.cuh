@@ -137,7 +137,7 @@ __device__ __forceinline__ void solute_geq(float C, float ux, float uy, float (&
   }
   if (Q == 9) {
     // the rounded D2Q9 weights would bias sum g_eq and sum g_eq e (see
-    // equilibrium_pairs); restore C and C u
+    // equilibrium in lbarith.cuh); restore C and C u
     const float mx = geq[1] - geq[3] + geq[5] - geq[6] - geq[7] + geq[8];
     const float my = geq[2] - geq[4] + geq[5] + geq[6] - geq[7] - geq[8];
     const float cx = 0.5f * (C * ux - mx), cy = 0.5f * (C * uy - my);
