@@ -33,6 +33,7 @@ struct lb_batch {
   int4 *d_tiles = nullptr;
   unsigned int *d_counters = nullptr;
   unsigned int *d_tick = nullptr;
+  bool odd = false;  // the last call ended with an odd number of launches
   std::vector<BatchLat> h_lat;
   int shape = 0, dynamic = 1, order = 1;
   int ntiles = 0, grid = 0;
@@ -311,6 +312,13 @@ int lb_batch_iteration(lb_batch *b, int Nt, int use_graph) {
   BCK(cudaSetDevice(b->device));
   int rc = sync_descs(b);
   if (rc != LB_OK) return rc;
+  if (b->odd && Nt > 0) {
+    // every call starts with parity 0: its work counter is cleared (the last
+    // launch, of parity 0 too, used it) and takes up the launch number
+    BCK(cudaMemsetAsync(b->d_counters, 0, sizeof(unsigned int), b->stream));
+    BCK(cudaMemcpyAsync(b->d_tick, b->d_tick + 1, sizeof(unsigned int), cudaMemcpyDeviceToDevice, b->stream));
+  }
+  if (Nt > 0) b->odd = Nt & 1;
   int done = 0;
   // poisoned members run without the graph (the poisoning is not captured)
   if (use_graph && !batch_poisoned(b)) {
