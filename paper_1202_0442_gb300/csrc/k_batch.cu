@@ -163,6 +163,18 @@ int batch_occupancy(int storage, int shape) {
   }
 }
 
+int launch_march_batch_f32(const MarchBatch &b, int parity, cudaStream_t s);
+int launch_march_batch_f16(const MarchBatch &b, int parity, cudaStream_t s);
+int launch_march_batch_bf16(const MarchBatch &b, int parity, cudaStream_t s);
+
+int launch_march_batch(int storage, const MarchBatch &b, int parity, cudaStream_t s) {
+  switch (storage) {
+    case ST_FP16: return launch_march_batch_f16(b, parity, s);
+    case ST_BF16: return launch_march_batch_bf16(b, parity, s);
+    default: return launch_march_batch_f32(b, parity, s);
+  }
+}
+
 int launch_batch(int storage, const BatchLaunch &b, int parity, cudaStream_t s) {
   switch (storage) {
     case ST_FP16: return launch_s<__half>(b, parity, s);

@@ -444,12 +444,10 @@ int launch_march_f16(const MarchArgs &a, dim3 grid, dim3 block, cudaStream_t s);
 int launch_march_bf16(const MarchArgs &a, dim3 grid, dim3 block, cudaStream_t s);
 
 int launch_march(int storage, MarchArgs &a, int sms, cudaStream_t s) {
-  const Geometry &g = a.f.g;
-  // strips of equal width
-  const int n = (g.nx + MARCH_COLS - 1) / MARCH_COLS;
-  a.sw = ((g.nx + n - 1) / n + 1) & ~1;
+  const MarchLat &g = a.l;
+  a.sw = march_strip_width(g.nx);
   const int all = (g.nx + a.sw - 1) / a.sw;
-  const bool edges = a.f.nopen > 0;
+  const bool edges = a.op.nopen > 0;
   a.last = (all - 1) * a.sw;
   a.x0 = edges ? a.sw : 0;
   a.strips = edges ? std::max(all - 2, 0) : all;

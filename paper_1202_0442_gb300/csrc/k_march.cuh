@@ -21,6 +21,7 @@
 // unrolled once instead of twice (more register moves): 8.2.
 #pragma once
 
+#include "lbbatch.h"
 #include "lbcollide.cuh"
 #include "lbpdl.cuh"
 
@@ -52,11 +53,16 @@ template <> struct Pair<float> {
   }
   static __device__ __forceinline__ R keep(R v, bool a, bool b) { return mk2(a ? lo(v) : 0.f, b ? hi(v) : 0.f); }
   static __device__ __forceinline__ f2 val(R v) { return v; }
-  static __device__ __forceinline__ void st(float *p, unsigned o, R v) { *(unsigned long long *)(p + o) = v.v; }
+  static __device__ __forceinline__ void st(float *p, unsigned o, R v) {
+    asm volatile("st.global.b64 [%0], %1;" ::"l"(__cvta_generic_to_global(p + o)), "l"(v.v) : "memory");
+  }
 };
 
 struct Pair16 {
   using R = uint32_t;
+  static __device__ __forceinline__ void st32(void *p, uint32_t v) {
+    asm volatile("st.global.b32 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "r"(v) : "memory");
+  }
   static __device__ __forceinline__ R left(R v) {
     return __byte_perm(__shfl_up_sync(0xffffffffu, v, 1), v, 0x5432);
   }
@@ -86,7 +92,7 @@ template <> struct Pair<__half> : Pair16 {
     const __half2 h = __floats2half2_rn(a, b);
     return *reinterpret_cast<const uint32_t *>(&h);
   }
-  static __device__ __forceinline__ void st(__half *p, unsigned o, R v) { *(uint32_t *)(p + o) = v; }
+  static __device__ __forceinline__ void st(__half *p, unsigned o, R v) { st32(p + o, v); }
 };
 
 template <> struct Pair<__nv_bfloat16> : Pair16 {
@@ -103,7 +109,7 @@ template <> struct Pair<__nv_bfloat16> : Pair16 {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<const uint32_t *>(&h);
   }
-  static __device__ __forceinline__ void st(__nv_bfloat16 *p, unsigned o, R v) { *(uint32_t *)(p + o) = v; }
+  static __device__ __forceinline__ void st(__nv_bfloat16 *p, unsigned o, R v) { st32(p + o, v); }
 };
 
 // the pulled populations of a row's pairs: m2, m5, m6 from the row below, z
@@ -148,21 +154,21 @@ struct LaneOpen {
   int rows;         // its rule depends on the row (bit 0: a, bit 1: b)
 };
 
-__device__ __forceinline__ void lane_open(const FluidArgs &p, const int (&x)[2], float sc, LaneOpen &L) {
+__device__ __forceinline__ void lane_open(const MarchLat &p, const MarchOpen &op, const int (&x)[2], float sc, LaneOpen &L) {
   int on = 0, rows = 0;
 #pragma unroll
   for (int j = 0; j < 2; j++) {
     float m = 0.f, b = 0.f;
     int a0 = 1, a1 = 0;
 #pragma unroll 1
-    for (int k = 0; k < p.nopen; k++) {
-      const int wall = span_wall(p.span[k]);
-      if (x[j] != (wall == 0 ? 0 : p.g.nx - 1) || a0 <= a1) continue;
-      if (!opening_mb(p.span[k], p.rule[k], 0, 0, p.rho_ref[0], sc, m, b)) continue;
-      a0 = p.span[k].wa0 >> 2;
-      a1 = p.span[k].a1;
+    for (int k = 0; k < op.nopen; k++) {
+      const int wall = span_wall(op.span[k]);
+      if (x[j] != (wall == 0 ? 0 : p.nx - 1) || a0 <= a1) continue;
+      if (!opening_mb(op.span[k], op.rule[k], 0, 0, p.rho_ref, sc, m, b)) continue;
+      a0 = op.span[k].wa0 >> 2;
+      a1 = op.span[k].a1;
       on |= (1 | wall << 2) << j;
-      if ((p.rule[k].bits & 7) == OPEN_POISEUILLE) rows |= 1 << j;
+      if ((op.rule[k].bits & 7) == OPEN_POISEUILLE) rows |= 1 << j;
     }
     L.m[j] = m;
     L.b[j] = b;
@@ -174,16 +180,17 @@ __device__ __forceinline__ void lane_open(const FluidArgs &p, const int (&x)[2],
 }
 
 // the opening rules of the lane's nodes in row y
-__device__ __forceinline__ void open_pair(const FluidArgs &p, const LaneOpen &L, int y, float sc, f2 (&v)[9]) {
+__device__ __forceinline__ void open_pair(const MarchLat &p, const MarchOpen &op, const LaneOpen &L, int y, float sc,
+                                          f2 (&v)[9]) {
   const int in = L.on & ((y >= L.a0[0] && y <= L.a1[0] ? 5 : 0) | (y >= L.a0[1] && y <= L.a1[1] ? 10 : 0));
   f2 m = mk2(L.m[0], L.m[1]), b = mk2(L.b[0], L.b[1]);
   if (in & L.rows) {
     float mm[2] = {lo(m), hi(m)}, bb[2] = {lo(b), hi(b)};
 #pragma unroll 1
-    for (int k = 0; k < p.nopen; k++) {
-      const int wall = span_wall(p.span[k]);
+    for (int k = 0; k < op.nopen; k++) {
+      const int wall = span_wall(op.span[k]);
       float mk = 0.f, bk = 0.f;
-      opening_mb(p.span[k], p.rule[k], 0, y, p.rho_ref[0], sc, mk, bk);
+      opening_mb(op.span[k], op.rule[k], 0, y, p.rho_ref, sc, mk, bk);
 #pragma unroll
       for (int j = 0; j < 2; j++)
         if ((L.rows >> j & 1) && (L.on >> (2 + j) & 1) == wall) {
@@ -209,21 +216,21 @@ __device__ __forceinline__ void open_pair(const FluidArgs &p, const LaneOpen &L,
 // the collision of two nodes (columns xa and xb of row y), rounded to the
 // storage format; the same operations as collide_store on each
 template <class S, bool PM, int SR, int RX, bool OPEN, class R>
-__device__ __forceinline__ void collide_pair(const FluidArgs &p, const LaneOpen &L, int xa, int xb, int y, uint32_t seed,
+__device__ __forceinline__ void collide_pair(const MarchLat &p, const MarchOpen *op, const LaneOpen &L, int xa, int xb, int y, uint32_t seed,
                                              const R (&h)[9], R (&o)[9], f2 *fields = nullptr) {
   using P = Pair<S>;
   constexpr bool FOLD = Store<S>::kScaled;
   f2 v[9];
 #pragma unroll
   for (int i = 0; i < 9; i++) v[i] = P::val(h[i]);
-  if (OPEN) open_pair(p, L, y, FOLD ? p.scale : 1.0f, v);
+  if (OPEN) open_pair(p, *op, L, y, FOLD ? p.scale : 1.0f, v);
   Node1<f2> n;
-  moments1<f2, PM, FOLD>(v, p.rho_ref[0], p.inv_scale, n);
-  n.Fx = vfma(n.rho, vset<f2>(p.ax[0]), vset<f2>(p.fx[0]));
-  n.Fy = vfma(n.rho, vset<f2>(p.ay[0]), vset<f2>(p.fy[0]));
-  shift1<f2, PM>(p.tau[0], n);
+  moments1<f2, PM, FOLD>(v, p.rho_ref, p.inv_scale, n);
+  n.Fx = vfma(n.rho, vset<f2>(p.ax), vset<f2>(p.fx));
+  n.Fy = vfma(n.rho, vset<f2>(p.ay), vset<f2>(p.fy));
+  shift1<f2, PM>(p.tau, n);
   f2 heq[9];
-  equilibrium1<f2, FOLD>(n, p.scale, p.wa[0], p.wd[0], heq);
+  equilibrium1<f2, FOLD>(n, p.scale, p.wa, p.wd, heq);
   if (fields) {
     const f2 half = vset<f2>(0.5f);
     fields[0] = n.drho;
@@ -231,14 +238,14 @@ __device__ __forceinline__ void collide_pair(const FluidArgs &p, const LaneOpen 
     fields[2] = vadd(n.jy, vfma(half, n.Fy, n.jyl));
     fields[3] = equilibrium_sum(heq, FOLD ? p.inv_scale : 1.0f);
   }
-  relax<RX>(v, heq, p.omega[0], p.keep);
+  relax<RX>(v, heq, p.omega, p.keep);
   if constexpr (sizeof(S) == 4) {
 #pragma unroll
     for (int i = 0; i < 9; i++) o[i] = v[i];
   } else if constexpr (SR == 2) {
     // the dithers of collide_store: a hash per node, one step of a linear
     // congruential sequence per two directions
-    uint32_t ra = rnd(seed, y * p.g.pitch + xa, 0, 0), rb = rnd(seed, y * p.g.pitch + xb, 0, 0);
+    uint32_t ra = rnd(seed, y * p.pitch + xa, 0, 0), rb = rnd(seed, y * p.pitch + xb, 0, 0);
 #pragma unroll
     for (int i = 0; i < 8; i += 2) {
       ra = ra * 1664525u + 1013904223u;
@@ -260,19 +267,17 @@ __device__ __forceinline__ void collide_pair(const FluidArgs &p, const LaneOpen 
 // two iterations of rows [ys, ye) of the columns [X0, X1), by one
 // warp; OPEN: the strip's columns or their halo touch a wall with openings
 template <class S, bool PM, int SR, int RX, bool FIELDS, bool OPEN, int U>
-__device__ __forceinline__ void march_strip(const MarchArgs &a, LaneOpen *lanes, int X0, int X1, int ys, int ye) {
+__device__ __forceinline__ void march_strip(const MarchLat &p, const MarchOpen *op, LaneOpen *lanes, int X0, int X1, int ys, int ye) {
   using P = Pair<S>;
   using R = typename P::R;
-  const FluidArgs &p = a.f;
-  const Geometry &g = p.g;
   const int lane = threadIdx.x;
   const int xa = X0 - 2 + 2 * lane;  // the lane's columns xa, xa + 1
   // wrapped columns; lanes past the strip's halo repeat its last pair
   const int xc = min(xa, (X1 + 1) & ~1);
-  const int wa = wrapi(xc, g.nx), wb = wrapi(xc + 1, g.nx);
+  const int wa = wrapi(xc, p.nx), wb = wrapi(xc + 1, p.nx);
   const bool wide = __all_sync(0xffffffffu, !(wa & 1) && wb == wa + 1);
-  LaneOpen &L = lanes[threadIdx.y * 32 + lane];
-  if (OPEN) lane_open(p, {wa, wb}, Store<S>::kScaled ? p.scale : 1.0f, L);
+  LaneOpen &L = lanes[OPEN ? threadIdx.y * 32 + lane : 0];
+  if (OPEN) lane_open(p, *op, {wa, wb}, Store<S>::kScaled ? p.scale : 1.0f, L);
   const bool mine = xa >= X0 && xa < X1;
   const bool bcol = xa + 1 < X1;  // an odd lattice's last pair ends in row padding
   // lanes that share the lane's 32-byte sector
@@ -280,12 +285,12 @@ __device__ __forceinline__ void march_strip(const MarchArgs &a, LaneOpen *lanes,
   const int gs = lane - ((xa >> 1) & (LPS - 1));
   constexpr unsigned GM = (1u << LPS) - 1u;
   const unsigned sector = gs >= 0 ? GM << gs : GM >> -gs;
-  const unsigned Pl = (unsigned)g.plane;
+  const unsigned Pl = p.plane;
   const S *fin = (const S *)p.fin;
   S *fout = (S *)p.fout;
 
   auto load = [&](int row, R(&v)[9], uint32_t &c) {
-    const unsigned ro = (unsigned)row * (unsigned)g.pitch;
+    const unsigned ro = (unsigned)row * (unsigned)p.pitch;
     const unsigned oa = ro + wa, ob = ro + wb;
     if (wide) {
       c = __ldg((const uint32_t *)(p.nbc + oa));
@@ -301,7 +306,7 @@ __device__ __forceinline__ void march_strip(const MarchArgs &a, LaneOpen *lanes,
     constexpr uint32_t SELF = 1u << NBPOS(0, 0);
     const bool fa = mine && !(c & SELF), fb = mine && bcol && !(c & (SELF << 16));
     const unsigned busy = __ballot_sync(0xffffffffu, fa || fb);
-    const unsigned o = (unsigned)row * (unsigned)g.pitch + (unsigned)xa;
+    const unsigned o = (unsigned)row * (unsigned)p.pitch + (unsigned)xa;
     if (mine && (busy & sector)) {
       if (fa && fb) {
 #pragma unroll
@@ -313,11 +318,11 @@ __device__ __forceinline__ void march_strip(const MarchArgs &a, LaneOpen *lanes,
       }
     }
   };
-  auto next = [&](int y) { return y + 1 == g.ny ? 0 : y + 1; };
+  auto next = [&](int y) { return y + 1 == p.ny ? 0 : y + 1; };
 
   R z[9], q[9], h[9], m2, m5, m6;
   uint32_t cz, cq, cl = 0;
-  int yz = wrapi(ys - 2, g.ny);
+  int yz = wrapi(ys - 2, p.ny);
   load(yz, z, cz);
   m2 = z[2];
   m5 = z[5];
@@ -345,18 +350,18 @@ __device__ __forceinline__ void march_strip(const MarchArgs &a, LaneOpen *lanes,
     yq = next(yq);
     if (k < ye) load(yq, q, cq);
     R o[9];
-    collide_pair<S, PM, SR, RX, OPEN>(p, L, wa, wb, y, p.sr_seed, h, o);
+    collide_pair<S, PM, SR, RX, OPEN>(p, op, L, wa, wb, y, p.seed, h, o);
     if (k > ys) {
       // the second iteration of row k - 1
       const int y2 = k - 1;
       R h2[9], o2[9];
       f2 fl[NFIELD];
       gather<S>(s2, s5, s6, s, o[4], o[7], o[8], cl, h2);
-      collide_pair<S, PM, SR, RX, OPEN>(p, L, wa, wb, y2, a.sr_seed2, h2, o2, FIELDS ? fl : nullptr);
+      collide_pair<S, PM, SR, RX, OPEN>(p, op, L, wa, wb, y2, p.seed2, h2, o2, FIELDS ? fl : nullptr);
       store(y2, o2, cl);
       if (FIELDS) {
         constexpr uint32_t SELF = 1u << NBPOS(0, 0);
-        const unsigned at = (unsigned)y2 * (unsigned)g.pitch + (unsigned)xa;
+        const unsigned at = (unsigned)y2 * (unsigned)p.pitch + (unsigned)xa;
 #pragma unroll
         for (int i = 0; i < NFIELD; i++) {
           if (mine && !(cl & SELF)) p.fields[(size_t)i * Pl + at] = lo(fl[i]);
@@ -381,37 +386,77 @@ template <class S, bool PM, int SR, int RX, bool FIELDS>
 __global__ void __launch_bounds__(128, 4) k_march(const MarchArgs a) {
   __shared__ LaneOpen lanes[128];
   dep_wait();
-  const Geometry &g = a.f.g;
+  const MarchLat &g = a.l;
   const int b = (int)blockIdx.x - a.eb;
   if (b < 0) {
     const int e = blockIdx.x * blockDim.y + threadIdx.y;
     const int X0 = (e & 1) * a.last, ys = (e >> 1) * a.eseg;
     if (ys < g.ny && !((e & 1) && a.last == 0))
-      march_strip<S, PM, SR, RX, FIELDS, true, 1>(a, lanes, X0, min(X0 + a.sw, g.nx), ys, min(ys + a.eseg, g.ny));
+      march_strip<S, PM, SR, RX, FIELDS, true, 1>(a.l, &a.op, lanes, X0, min(X0 + a.sw, g.nx), ys, min(ys + a.eseg, g.ny));
   } else {
     const int row = b / a.bx, strip = (b - row * a.bx) * blockDim.y + threadIdx.y;
     if (strip < a.strips) {
       const int X0 = a.x0 + strip * a.sw, ys = row * a.seg;
-      march_strip<S, PM, SR, RX, FIELDS, false, 2>(a, lanes, X0, min(X0 + a.sw, g.nx), ys, min(ys + a.seg, g.ny));
+      march_strip<S, PM, SR, RX, FIELDS, false, 2>(a.l, &a.op, lanes, X0, min(X0 + a.sw, g.nx), ys, min(ys + a.seg, g.ny));
     }
   }
+}
+
+// the same for the lattices of a batch: a task per warp, the lattice's
+// parameters in shared memory (the loop not unrolled: with them in general
+// registers the copy spills 188 B instead of 60; 256 lattices FP32 192 us
+// per iteration against 200; k_batch takes 280, as does a launch per
+// iteration of this kernel's bytes, 72 B per node).  The launch numbers of its two iterations
+// are those of k_batch (tick), so the dithers do not depend on which of the
+// two kernels advances an iteration.
+template <class S, bool PM, int SR>
+__global__ void __launch_bounds__(128, 4) k_march_batch(const MarchBatch b, int parity) {
+  __shared__ MarchBatchLat lats[4];
+  const unsigned int launch_no = b.tick[parity];
+  if (blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) {
+    b.tick[1 - parity] = launch_no + 2u;
+    b.counters[1 - parity] = 0;
+  }
+  const int k = blockIdx.x * 4 + threadIdx.y;
+  if (k >= b.ntasks) return;
+  const int4 t = __ldg(b.tasks + k);
+  MarchBatchLat &m = lats[threadIdx.y];
+  static_assert(sizeof(MarchBatchLat) % 4 == 0 && sizeof(MarchBatchLat) <= 128 + 32, "two words per lane");
+  const uint32_t *src = reinterpret_cast<const uint32_t *>(b.lat + t.x);
+  for (int i = threadIdx.x; i < (int)(sizeof(MarchBatchLat) / 4); i += 32) reinterpret_cast<uint32_t *>(&m)[i] = __ldg(src + i);
+  __syncwarp();
+  if (threadIdx.x == 0) {
+    m.l.seed = mix32(launch_no * 0x9e3779b9u + (uint32_t)t.x);
+    m.l.seed2 = mix32((launch_no + 1u) * 0x9e3779b9u + (uint32_t)t.x);
+  }
+  __syncwarp();
+  march_strip<S, PM, SR, 0, false, false, 1>(m.l, nullptr, nullptr, t.y, min(t.y + m.sw, m.l.nx), t.z,
+                                             min(t.z + t.w, m.l.ny));
+}
+
+template <class S, int SR>
+int launch_march_batch_t(const MarchBatch &b, int parity, cudaStream_t s) {
+  const dim3 grid((b.ntasks + 3) / 4), block(32, 4);
+  if (b.pm) k_march_batch<S, true, SR><<<grid, block, 0, s>>>(b, parity);
+  else k_march_batch<S, false, SR><<<grid, block, 0, s>>>(b, parity);
+  return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
 template <class S, int SR, int RX>
 int launch_march_r(const MarchArgs &a, dim3 grid, dim3 block, cudaStream_t s) {
   cudaError_t e;
-  if (a.f.fields)
-    e = a.f.pm ? launch_pdl(k_march<S, true, SR, RX, true>, grid, block, 0, s, a)
+  if (a.l.fields)
+    e = a.pm ? launch_pdl(k_march<S, true, SR, RX, true>, grid, block, 0, s, a)
                : launch_pdl(k_march<S, false, SR, RX, true>, grid, block, 0, s, a);
   else
-    e = a.f.pm ? launch_pdl(k_march<S, true, SR, RX, false>, grid, block, 0, s, a)
+    e = a.pm ? launch_pdl(k_march<S, true, SR, RX, false>, grid, block, 0, s, a)
                : launch_pdl(k_march<S, false, SR, RX, false>, grid, block, 0, s, a);
   return e == cudaSuccess ? 1 : -1;
 }
 
 template <class S, int SR>
 int launch_march_t(const MarchArgs &a, dim3 grid, dim3 block, cudaStream_t s) {
-  return a.f.omega[0] >= 1.0f ? launch_march_r<S, SR, 1>(a, grid, block, s) : launch_march_r<S, SR, 2>(a, grid, block, s);
+  return a.l.omega >= 1.0f ? launch_march_r<S, SR, 1>(a, grid, block, s) : launch_march_r<S, SR, 2>(a, grid, block, s);
 }
 
 }  // namespace

@@ -4,7 +4,11 @@
 namespace lbk {
 
 int launch_march_bf16(const MarchArgs &a, dim3 grid, dim3 block, cudaStream_t s) {
-  return a.f.sr_seed ? launch_march_t<__nv_bfloat16, 2>(a, grid, block, s) : launch_march_t<__nv_bfloat16, 1>(a, grid, block, s);
+  return a.sr ? launch_march_t<__nv_bfloat16, 2>(a, grid, block, s) : launch_march_t<__nv_bfloat16, 1>(a, grid, block, s);
+}
+
+int launch_march_batch_bf16(const MarchBatch &b, int parity, cudaStream_t s) {
+  return b.sr ? launch_march_batch_t<__nv_bfloat16, 2>(b, parity, s) : launch_march_batch_t<__nv_bfloat16, 1>(b, parity, s);
 }
 
 }  // namespace lbk

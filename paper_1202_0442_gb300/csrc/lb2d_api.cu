@@ -837,15 +837,47 @@ bool march_ok(const lb_ctx *ctx) {
   return (int64_t)ctx->nx * ctx->ny >= 320000 && ctx->nx * 5 >= strips * 64 * 3;
 }
 
+void march_lattice(const FluidArgs &f, MarchLat &l) {
+  l.fin = f.fin;
+  l.fout = f.fout;
+  l.nbc = f.nbc;
+  l.fields = f.fields;
+  l.nx = f.g.nx;
+  l.ny = f.g.ny;
+  l.pitch = f.g.pitch;
+  l.plane = (unsigned)f.g.plane;
+  l.rho_ref = f.rho_ref[0];
+  l.scale = f.scale;
+  l.inv_scale = f.inv_scale;
+  l.tau = f.tau[0];
+  l.omega = f.omega[0];
+  l.keep = f.keep;
+  l.wa = f.wa[0];
+  l.wd = f.wd[0];
+  l.fx = f.fx[0];
+  l.fy = f.fy[0];
+  l.ax = f.ax[0];
+  l.ay = f.ay[0];
+  l.seed = f.sr_seed;
+}
+
 // two iterations in one launch; fields: node fields after the second
 int two_steps(lb_ctx *ctx, bool fields) {
   NvtxRange range("step");
   ctx->t += 1;
   const int nxt = 1 - ctx->cur;
-  MarchArgs a{};
-  a.f = fluid_args(ctx, fields);
+  const FluidArgs f = fluid_args(ctx, fields);
   ctx->t += 1;
-  a.sr_seed2 = ctx->sr ? (uint32_t)step_word(ctx->t) | 1u : 0u;
+  MarchArgs a{};
+  march_lattice(f, a.l);
+  a.l.seed2 = (uint32_t)step_word(ctx->t) | 1u;
+  a.op.nopen = f.nopen;
+  for (int k = 0; k < f.nopen; k++) {
+    a.op.span[k] = f.span[k];
+    a.op.rule[k] = f.rule[k];
+  }
+  a.pm = f.pm;
+  a.sr = ctx->sr ? 1 : 0;
   if (ctx->debug & LB_DEBUG_POISON) TRY(poison_outputs(ctx, nxt, fields));
   LAUNCH(launch_march(ctx->storage, a, ctx->sms, ctx->stream));
   ctx->cur = nxt;

@@ -5,6 +5,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "lbint.h"
+
 namespace lbk {
 
 // one lattice of a batch (periodic, one component, body forces only)
@@ -32,10 +34,27 @@ struct BatchLaunch {
                           // stochastic-rounding dither changes every launch
 };
 
+// two iterations of every lattice per launch (k_march.cuh), one strip and
+// segment of rows per warp
+struct MarchBatchLat {
+  MarchLat l;
+  int sw;                // columns of a strip
+  int pad;
+};
+
+struct MarchBatch {
+  const MarchBatchLat *lat; // device array for this parity's buffers
+  const int4 *tasks;        // device array of (lattice, first column, first row, rows)
+  int ntasks;
+  int pm, sr;               // of every lattice
+  unsigned int *counters, *tick;  // as BatchLaunch
+};
+
 constexpr int BATCH_SHAPES = 6;
 int batch_shape_tx(int shape);
 int batch_shape_ty(int shape);
 int batch_occupancy(int storage, int shape);
+int launch_march_batch(int storage, const MarchBatch &b, int parity, cudaStream_t s);
 int launch_batch(int storage, const BatchLaunch &b, int parity, cudaStream_t s);
 
 }  // namespace lbk

@@ -111,12 +111,35 @@ struct FluidArgs {
   int edge_x, edge_y;
 };
 
-// two iterations of a whole single-component lattice in one pass
-// (k_march.cuh): f.sr_seed dithers the first, sr_seed2 the second
+// one lattice of k_march (two iterations of a whole single-component
+// lattice in one pass, k_march.cuh)
+struct MarchLat {
+  const void *fin;
+  void *fout;
+  const uint16_t *nbc;
+  float *fields;      // node fields after the second iteration, or nullptr
+  int nx, ny, pitch;
+  unsigned plane;
+  float rho_ref, scale, inv_scale, tau, omega, keep, wa, wd, fx, fy, ax, ay;  // as FluidArgs
+  uint32_t seed, seed2;  // of the two iterations' rounding dithers
+};
+
+struct MarchOpen {
+  int nopen;
+  OpenSpan span[MAX_OPEN];
+  OpenRule rule[MAX_OPEN];
+};
+
 constexpr int MARCH_COLS = 60;
+// columns of a strip: equal strips, an even width
+inline int march_strip_width(int nx) {
+  const int n = (nx + MARCH_COLS - 1) / MARCH_COLS;
+  return ((nx + n - 1) / n + 1) & ~1;
+}
 struct MarchArgs {
-  FluidArgs f;
-  uint32_t sr_seed2;
+  MarchLat l;
+  MarchOpen op;
+  int pm, sr;              // exact momentum pairs; stochastic rounding
   int sw;                  // columns a warp advances (even, <= MARCH_COLS)
   int x0, strips, seg, bx; // the strips without an opening: first column,
                            // their number, rows per warp, blocks per row

@@ -70,3 +70,28 @@ def test_march_equals_single_iterations(nx, ny, openings, storage):
             assert np.array_equal(x, y)
         assert np.array_equal(a.fields()[3], b.fields()[3])
     assert b.launch_count() < a.launch_count() - 6
+
+
+@pytest.mark.parametrize("storage", list(STORAGE))
+def test_batch_by_pairs_equals_single_iterations(storage):
+    """The batched launch's pairs of iterations against its single ones (calls
+    of one iteration), bit for bit, over lattices of uneven sizes (one strip,
+    odd sides, fewer rows than a segment, either form of the relaxation)."""
+    st, kw = STORAGE[storage]
+    sizes = [(64, 512), (333, 190), (512, 480), (61, 31), (96, 5), (1, 1), (301, 299)]
+    taus = [0.6, 1.5, 0.8, 1.0, 0.9, 0.7, 1.2]
+    out = []
+    for calls in ([11, 24], [1] * 35):
+        lats = []
+        for k, ((nx, ny), tau) in enumerate(zip(sizes, taus)):
+            w = _workload(nx, ny, None)
+            w.tau = (tau,)
+            lats.append(lb2d.from_workload(w, st, thermo=1 << 30, **kw))
+        b = lb2d.Batch(lats)
+        for n in calls:
+            b.iteration(n)
+        out.append([(lt.populations(), lt.current_buffer()) for lt in lats])
+        launches = b.launch_count()
+    assert launches == 35
+    for (x, i), (y, j) in zip(*out):
+        assert i == j and np.array_equal(x, y)
