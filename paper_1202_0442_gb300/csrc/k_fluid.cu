@@ -476,6 +476,19 @@ int launch_march(int storage, MarchArgs &a, int sms, cudaStream_t s) {
   }
 }
 
+int launch_tile_f32(const TileArgs &a, dim3 grid, cudaStream_t s);
+int launch_tile_f16(const TileArgs &a, dim3 grid, cudaStream_t s);
+int launch_tile_bf16(const TileArgs &a, dim3 grid, cudaStream_t s);
+
+int launch_tile(int storage, const TileArgs &a, cudaStream_t s) {
+  const dim3 grid((a.l.nx + a.tw - 1) / a.tw, (a.l.ny + a.th - 1) / a.th);
+  switch (storage) {
+    case ST_FP16: return launch_tile_f16(a, grid, s);
+    case ST_BF16: return launch_tile_bf16(a, grid, s);
+    default: return launch_tile_f32(a, grid, s);
+  }
+}
+
 int launch_nbcode(const uint32_t *mask, uint16_t *nbc, const Geometry &g, cudaStream_t s, int r0, int r1) {
   if (r1 < 0) r1 = g.ny;
   if (r1 <= r0) return 0;

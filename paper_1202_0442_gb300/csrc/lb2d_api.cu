@@ -817,24 +817,63 @@ int one_step(lb_ctx *ctx, bool fields) {
   return LB_OK;
 }
 
-// whether k_march advances the lattice, two iterations per launch: a whole
-// single-component noslip lattice with body forces and velocity or density
-// openings (at most one on each x wall), the kernel not chosen by the
-// caller.  Below some 300 K nodes its few rows per warp are a serial chain
-// that the one-iteration kernel does not have (porous FP32: 512^2 3.8 us per
-// iteration either way, 256^2 3.5 against 2.2; 600 K nodes in BF16 6.7
-// against 8.4, 1024^2 7.8 against 10.2); and a width that fills the strips
-// badly leaves lanes idle.
-bool march_ok(const lb_ctx *ctx) {
+// whether the kernels that advance several iterations per launch (k_march,
+// k_tile) serve the lattice: a whole single-component noslip lattice with
+// body forces and velocity or density openings (at most one on each x
+// wall), the kernel not chosen by the caller
+bool several_ok(const lb_ctx *ctx) {
   if (ctx->nc != 1 || ctx->sc || ctx->qs || ctx->bstyle != 0 || ctx->rank >= 0 || ctx->kernel != 0 || ctx->ads[0])
     return false;
   int walls = 0;
   for (const Opening &o : ctx->open) {
-    if (o.style[0] == OPEN_GRADIENT || o.wall > 1 || (walls >> o.wall & 1)) return false;
+    if (o.style[0] == OPEN_GRADIENT || o.wall > 1 || ctx->nx < 4 || (walls >> o.wall & 1)) return false;
     walls |= 1 << o.wall;
   }
+  return true;
+}
+
+// Two iterations per launch (k_march) for large lattices.  Below some 300 K
+// nodes its few rows per warp are a serial chain that the one-iteration
+// kernel does not have (porous FP32: 512^2 3.8 us per iteration either way,
+// 256^2 3.5 against 2.2; 600 K nodes in BF16 6.7 against 8.4, 1024^2 7.8
+// against 10.2); and a width that fills the strips badly leaves lanes idle.
+bool march_ok(const lb_ctx *ctx) {
   const int strips = (ctx->nx + MARCH_COLS - 1) / MARCH_COLS;
   return (int64_t)ctx->nx * ctx->ny >= 320000 && ctx->nx * 5 >= strips * 64 * 3;
+}
+
+// The tiles of k_tile: for T iterations per launch the grid of at most one
+// block per SM whose tiles with their halo are the smallest, and the T that
+// costs the least per iteration, if that is less than the one-iteration
+// kernel's (T = 1).  Costs in us, from timings with T = 2..12: a launch 1.8 and
+// 3 per 1000 nodes read, an iteration 0.4 and 0.65 per round of the block's
+// threads over its pairs of nodes (porous FP32: 256^2 T = 5 1.73 per iteration,
+// T = 8 2.00, single 2.32; 400^2 T = 6 2.80, T = 3 3.78, single 3.09; 512^2
+// 3.90 against 3.83: not taken); the one-iteration kernel 1.75 and 8 per
+// million nodes.
+void plan_tiles(lb_ctx *ctx) {
+  ctx->tile_steps = 1;
+  double best = 1.75 + 8e-6 * (double)ctx->nx * ctx->ny;
+  for (int T = 2; T <= TILE_STEPS; T++) {
+    int64_t least = TILE_NODES + 1;
+    for (int bx = 1; bx <= ctx->sms && bx <= ctx->nx; bx++) {
+      const int by = std::min(ctx->sms / bx, ctx->ny);
+      const int tw = (ctx->nx + bx - 1) / bx, th = (ctx->ny + by - 1) / by;
+      const int64_t nodes = (int64_t)(tw + 2 * T) * ((th + 2 * T + 1) & ~1);
+      if (nodes < least) {
+        least = nodes;
+        ctx->tile_w[T] = tw;
+        ctx->tile_h[T] = th;
+      }
+    }
+    if (least > TILE_NODES) break;
+    const double rounds = (double)((least / 2 + TILE_THREADS - 1) / TILE_THREADS);
+    const double cost = (1.8 + 3e-3 * (double)least) / T + 0.4 + 0.65 * rounds;
+    if (cost < best) {
+      best = cost;
+      ctx->tile_steps = T;
+    }
+  }
 }
 
 void march_lattice(const FluidArgs &f, MarchLat &l) {
@@ -881,6 +920,47 @@ int two_steps(lb_ctx *ctx, bool fields) {
   if (ctx->debug & LB_DEBUG_POISON) TRY(poison_outputs(ctx, nxt, fields));
   LAUNCH(launch_march(ctx->storage, a, ctx->sms, ctx->stream));
   ctx->cur = nxt;
+  return LB_OK;
+}
+
+// T iterations of a small lattice in one launch; fields: node fields after
+// the last
+int tile_launch(lb_ctx *ctx, int T, bool fields) {
+  NvtxRange range("step");
+  const int nxt = 1 - ctx->cur;
+  const FluidArgs f = fluid_args(ctx, fields);
+  TileArgs a{};
+  march_lattice(f, a.l);
+  a.op.nopen = f.nopen;
+  for (int k = 0; k < f.nopen; k++) {
+    a.op.span[k] = f.span[k];
+    a.op.rule[k] = f.rule[k];
+  }
+  a.pm = f.pm;
+  a.sr = ctx->sr ? 1 : 0;
+  a.steps = T;
+  a.tw = ctx->tile_w[T];
+  a.th = ctx->tile_h[T];
+  a.t0 = ctx->t;
+  if (ctx->debug & LB_DEBUG_POISON) TRY(poison_outputs(ctx, nxt, fields));
+  LAUNCH(launch_tile(ctx->storage, a, ctx->stream));
+  ctx->t += T;
+  ctx->cur = nxt;
+  return LB_OK;
+}
+
+// n iterations by tiles: launches of equal length, their number odd or even
+// as n is, so that the current buffer alternates as documented
+int tile_steps(lb_ctx *ctx, int64_t n, bool fields) {
+  int64_t launches = (n + ctx->tile_steps - 1) / ctx->tile_steps;
+  if ((launches ^ n) & 1) launches++;
+  while (launches > 0) {
+    const int T = (int)((n + launches - 1) / launches);
+    const bool last = launches == 1;
+    TRY(T >= 2 ? tile_launch(ctx, T, last && fields) : one_step(ctx, last && fields));
+    n -= T;
+    launches--;
+  }
   return LB_OK;
 }
 
@@ -1662,7 +1742,8 @@ int lb_iteration(lb_ctx *ctx, int Nt) {
   if (ctx->rank >= 0 && ctx->py > 1 && Nt > 1)
     return ctx->fail(LB_E_ORDER, "a slab of a lattice split into %d advances one iteration per call, its halo "
                      "rows exchanged between calls", ctx->py);
-  const bool march = march_ok(ctx);
+  const bool several = several_ok(ctx), march = several && march_ok(ctx);
+  if (several && !march && !ctx->tile_steps) plan_tiles(ctx);
   for (int k = 0; k < Nt;) {
     // iterations up to the next one whose end the host looks at
     int64_t n = Nt - k;
@@ -1674,6 +1755,7 @@ int lb_iteration(lb_ctx *ctx, int Nt) {
     // by twos an even number of times, so that the current buffer
     // alternates with the iterations as documented
     for (int64_t j = march ? n / 4 * 4 : 0; j > 0; j -= 2) TRY(two_steps(ctx, ctx->t + 2 == end && (thermo || out)));
+    if (several && !march && ctx->tile_steps > 1 && n > 2) TRY(tile_steps(ctx, n, thermo || out));
     while (ctx->t < end) {
       TRY(one_step(ctx, ctx->t + 1 == end && (thermo || out)));
       if (ctx->rank >= 0 && ctx->py == 1) TRY(exchange_slabs(&ctx, 1));

@@ -125,6 +125,10 @@ struct lb_ctx {
   int *errw = nullptr;   // device error word of the TMA kernel
   long long wait_limit = -1;  // TMA kernel's wait limit in clock cycles (-1: its default)
   int sms = 0;
+  // k_tile: nodes of a tile for each number of iterations per launch (tw 0:
+  // the lattice is too large), and the number that costs the least per
+  // iteration (0: not planned yet, 1: no tiles)
+  int tile_w[lbk::TILE_STEPS + 1] = {0}, tile_h[lbk::TILE_STEPS + 1] = {0}, tile_steps = 0;
   bool fields_valid = false;
   int64_t fields_step = -1;  // iteration whose end state the field planes hold
   lb_thermo_t thermo{};

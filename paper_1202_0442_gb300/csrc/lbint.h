@@ -147,6 +147,18 @@ struct MarchArgs {
                            // first column of the last one, rows per warp
 };
 
+// several iterations of a small lattice per launch (k_tile.cuh)
+constexpr int TILE_NODES = 2624;   // of a tile and its halo (230,912 B of shared memory)
+constexpr int TILE_THREADS = 512;
+constexpr int TILE_STEPS = 12;     // most iterations per launch
+struct TileArgs {
+  MarchLat l;
+  MarchOpen op;
+  int pm, sr;              // exact momentum pairs; stochastic rounding
+  int steps, tw, th;       // iterations; nodes of a tile
+  long long t0;            // iterations done before the launch
+};
+
 // gradient openings (after collision)
 struct GradArgs {
   Geometry g;
@@ -254,6 +266,7 @@ struct CopyRuns {
 // launchers (return the kernel count launched, or -1 on a launch error)
 int launch_fluid(int storage, int nc, bool sc, bool mass_exact, const FluidArgs &a, cudaStream_t s);
 int launch_march(int storage, MarchArgs &a, int sms, cudaStream_t s);
+int launch_tile(int storage, const TileArgs &a, cudaStream_t s);
 int launch_gradient(int storage, const GradArgs &a, cudaStream_t s);
 // fluid and solute iteration in one kernel (one component, no interforce,
 // no intersolute, no exact momentum pairs, streaming kernel)
