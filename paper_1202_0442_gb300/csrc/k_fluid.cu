@@ -206,6 +206,38 @@ __global__ void __launch_bounds__(32 * LOC_BY, 4 * 8 / LOC_BY) k_fluid_solute(co
   solute_node<Q>(sp, x, y, bits, u[0], u[1]);
 }
 
+// the pulled populations of both components of fluid node (x, y), with the
+// slip styles and the opening rules
+template <class S, bool SLIP, bool OPEN>
+__device__ __forceinline__ void pull_two(const FluidArgs &p, int x, int y, uint32_t bits, f2 (&h)[9]) {
+  const Geometry &g = p.g;
+  const S *a = (const S *)p.fin, *b = a + 9 * g.plane;
+  if constexpr (SLIP || OPEN) {
+    float f[2][9];
+    pull9<S>(a, g, x, y, bits, p.inv_scale, f[0]);
+    pull9<S>(b, g, x, y, bits, p.inv_scale, f[1]);
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+      if (SLIP && (bits & DIAG_BITS)) slip_fix<S>(p, c, c ? b : a, x, y, bits, p.inv_scale, f[c]);
+      if (OPEN) apply_opening_c(p, c, x, y, f[c]);
+    }
+#pragma unroll
+    for (int i = 0; i < 9; i++) h[i] = mk2(f[0][i], f[1][i]);
+  } else {
+    const int xm = x ? x - 1 : g.nx - 1, xp = (x + 1 == g.nx) ? 0 : x + 1;
+    const int ym = y ? y - 1 : g.ny - 1, yp = (y + 1 == g.ny) ? 0 : y + 1;
+    const int P = (int)g.plane;
+    const int r0 = y * g.pitch, rm = ym * g.pitch, rp = yp * g.pitch;
+    const int self = r0 + x;
+    const int src[9] = {self, r0 + xm, rm + x, r0 + xp, rp + x, rm + xm, rm + xp, rp + xp, rp + xm};
+#pragma unroll
+    for (int i = 0; i < 9; i++) {
+      const int k = (i && nb(bits, OPP(i))) ? OPP(i) * P + self : i * P + src[i];
+      h[i] = mk2(Store<S>::ld(a, k, p.inv_scale), Store<S>::ld(b, k, p.inv_scale));
+    }
+  }
+}
+
 // 32 x 8 tiles, 4 CTAs/SM: measured fastest of 32 x {4, 8, 16, 32} (the
 // barrier waits on fewer warps; the ring costs 33 % more pulls, from L1/L2)
 constexpr int SC_TX = 32, SC_TY = 8;
@@ -309,6 +341,69 @@ __global__ void __launch_bounds__(SC_TX *SC_TY, 4) k_fluid_sc(const FluidArgs p)
   collide_store_me<S, NC>(p, x, y, bits, h, F);
 }
 
+// k_fluid_sc for two components, both in every packed operation: one index
+// per population for both loads, one shared-memory word pair per neighbour,
+// and the collision of collide_store_two.  A solid node's staged density is
+// 0 (its deviation -rho_ref), so the force takes no test of the neighbours.
+// 64 registers without spills, as the scalar form had: 2048^2 FP32 154 us
+// per iteration against 175 (72 B per node and component: 89 at the copy
+// rate); still issue- and latency-bound at half the warps.  A warp per strip
+// that walks the rows (no ring, no barrier; 128 registers, 16 warps per SM)
+// took 195 to 260.
+template <class S, bool SLIP, bool OPEN>
+__global__ void __launch_bounds__(SC_TX *SC_TY, 4) k_fluid_sc2(const FluidArgs p) {
+  __shared__ f2 sd[SC_TY + 2][SC_TX + 2];
+  dep_wait();
+  const Geometry &g = p.g;
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int x0 = blockIdx.x * SC_TX, y0 = g.clo + blockIdx.y * SC_TY;
+  const int xr = x0 + tx, yr = y0 + ty;
+  const bool real = xr < g.nx && yr < g.chi;
+  const int x = wrapi(xr, g.nx), y = wrapi(yr, g.ny);
+  const uint32_t bits = __ldg(p.nbc + (size_t)y * g.pitch + x);
+  const bool solid = (bits >> 4) & 1u;
+  const f2 none = vsub(vset<f2>(0.f), both(p.rho_ref));
+  f2 h[9];
+  sd[ty + 1][tx + 1] = none;
+  if (!solid) {
+    pull_two<S, SLIP, OPEN>(p, x, y, bits, h);
+    sd[ty + 1][tx + 1] = density_sum(h);
+  }
+  // ring: 2 (TX + 2) + 2 TY slots, one thread each
+  const int tid = ty * SC_TX + tx;
+  constexpr int NRING = 2 * (SC_TX + 2) + 2 * SC_TY;
+  if (tid < NRING) {
+    int sx, sy;
+    if (tid < SC_TX + 2) { sx = tid; sy = 0; }
+    else if (tid < 2 * (SC_TX + 2)) { sx = tid - (SC_TX + 2); sy = SC_TY + 1; }
+    else if (tid < 2 * (SC_TX + 2) + SC_TY) { sx = 0; sy = tid - 2 * (SC_TX + 2) + 1; }
+    else { sx = SC_TX + 1; sy = tid - 2 * (SC_TX + 2) - SC_TY + 1; }
+    const int hx = wrapi(x0 + sx - 1, g.nx), hy = wrapi(y0 + sy - 1, g.ny);
+    const uint32_t hb = __ldg(p.nbc + (size_t)hy * g.pitch + hx);
+    f2 d = none;
+    if (!((hb >> 4) & 1u)) {
+      f2 hh[9];
+      pull_two<S, SLIP, OPEN>(p, hx, hy, hb, hh);
+      d = density_sum(hh);
+    }
+    sd[sy][sx] = d;
+  }
+  __syncthreads();
+  if (!real || solid) return;
+  // sum_i w_i rho(x + e_i) e_i from differences of opposite neighbours'
+  // deviations; F_c = -G rho_c sum_i w_i rho_o e_i takes the other
+  // component's sum
+  const f2(*n)[SC_TX + 2] = &sd[ty + 1];
+  const int cx = tx + 1;
+  const f2 ne = n[1][cx + 1], nw = n[1][cx - 1], se = n[-1][cx + 1], sw = n[-1][cx - 1];
+  const f2 ninth = vset<f2>(1.0f / 9.0f), t36 = vset<f2>(1.0f / 36.0f);
+  const f2 sx = vfma(ninth, vsub(n[0][cx + 1], n[0][cx - 1]), vmul(t36, vadd(vsub(ne, nw), vsub(se, sw))));
+  const f2 sy = vfma(ninth, vsub(n[1][cx], n[-1][cx]), vmul(t36, vadd(vsub(ne, se), vsub(nw, sw))));
+  const f2 d = n[0][cx];
+  const f2 a = vmul(vset<f2>(-p.G), vadd(both(p.rho_ref), d));
+  collide_store_two<S>(p, x, y, bits, h, d, vmul(a, swapped(sx)), vmul(a, swapped(sy)));
+}
+
 template <class S>
 __global__ void k_gradient(const GradArgs a) {
   // one thread per opening node of every gradient opening
@@ -383,10 +478,10 @@ int launch_fluid_t(int nc, bool sc, bool me, const FluidArgs &a, cudaStream_t s)
     const bool op = a.nopen > 0;
     if (a.slip) {
       if (nc == 1) launch_pdl(op ? k_fluid_sc<S, 1, true, true> : k_fluid_sc<S, 1, true, false>, grd, blk, 0, s, a);
-      else launch_pdl(op ? k_fluid_sc<S, 2, true, true> : k_fluid_sc<S, 2, true, false>, grd, blk, 0, s, a);
+      else launch_pdl(op ? k_fluid_sc2<S, true, true> : k_fluid_sc2<S, true, false>, grd, blk, 0, s, a);
     } else {
       if (nc == 1) launch_pdl(op ? k_fluid_sc<S, 1, false, true> : k_fluid_sc<S, 1, false, false>, grd, blk, 0, s, a);
-      else launch_pdl(op ? k_fluid_sc<S, 2, false, true> : k_fluid_sc<S, 2, false, false>, grd, blk, 0, s, a);
+      else launch_pdl(op ? k_fluid_sc2<S, false, true> : k_fluid_sc2<S, false, false>, grd, blk, 0, s, a);
     }
   } else {
     if (nc == 1) {

@@ -252,6 +252,121 @@ __device__ __forceinline__ void collide_store_me(const FluidArgs &p, int x, int 
   }
 }
 
+__device__ __forceinline__ f2 both(const float (&a)[2]) { return mk2(a[0], a[1]); }
+__device__ __forceinline__ f2 swapped(f2 a) { return mk2(hi(a), lo(a)); }
+
+// the rest population D - S of the mass-exact collision, rounded
+// stochastically in its last bit (rem: what h0 leaves out)
+__device__ __forceinline__ float last_bit(float h0, float rem, uint32_t word) {
+  if (rem == 0.f || h0 == 0.f) return h0;
+  const int step = ((rem > 0.f) == (h0 > 0.f)) ? 1 : -1;
+  const float nxt = __int_as_float(__float_as_int(h0) + step);
+  // |nxt - h0| is a power of two, so the quotient is exact up to the fast
+  // division's last bit: a probability, compared with a uniform variate
+  const float pr = __fdividef(fabsf(rem), fabsf(nxt - h0));
+  const float u01 = (float)(word >> 8) * (1.0f / 16777216.0f);
+  return u01 < pr ? nxt : h0;
+}
+
+// collide_store_me for two components, both in every packed operation (low
+// half: component 1), its error-free sums included.  h: the pulled
+// populations; d their sum; F: the interforce.
+template <class S>
+__device__ __forceinline__ void collide_store_two(const FluidArgs &p, int x, int y, uint32_t bits,
+                                                  const f2 (&h)[9], f2 d, f2 Fx, f2 Fy) {
+  const Geometry &g = p.g;
+  const int self = y * g.pitch + x;
+  const int hself = self + g.yoff * g.pitch;
+  const int P = (int)g.plane;
+  const f2 rho = vadd(both(p.rho_ref), d), tau = both(p.tau), om = both(p.omega);
+  f2 jx, jy;
+  momentum_sum(h, jx, jy);
+  Fx = vadd(Fx, vfma(rho, both(p.ax), both(p.fx)));
+  Fy = vadd(Fy, vfma(rho, both(p.ay), both(p.fy)));
+  constexpr uint32_t NB = 0x1efu;
+  if ((p.ads[0] | p.ads[1]) && (bits & NB)) {
+    float sx, sy;
+    wall_sum(bits, sx, sy);
+    const f2 a = vmul(mk2(p.ads[0] ? -p.Gads[0] : 0.f, p.ads[1] ? -p.Gads[1] : 0.f), rho);
+    Fx = vfma(a, vset<f2>(sx), Fx);
+    Fy = vfma(a, vset<f2>(sy), Fy);
+  }
+  // common velocity sum(j/tau) / sum(rho/tau): quotients by a reciprocal and
+  // one correction
+  const f2 nx = vmul(jx, om), ny = vmul(jy, om), nd = vmul(rho, om);
+  const f2 num = mk2(lo(nx) + hi(nx), lo(ny) + hi(ny)), den = vset<f2>(lo(nd) + hi(nd));
+  const f2 rd = vset<f2>(vrcp(lo(den)));
+  const f2 q = vmul(num, rd);
+  const f2 up = vfma(vfma(vsub(vset<f2>(0.f), q), den, num), rd, q);
+  const f2 tx = vmul(tau, Fx), ty = vmul(tau, Fy), ir = vrcp(rho);
+  const f2 upx = vset<f2>(lo(up)), upy = vset<f2>(hi(up));
+  const f2 mx = vfma(rho, upx, tx), my = vfma(rho, upy, ty);
+  f2 heq[9];
+  equilibrium(d, vfma(tx, ir, upx), vfma(ty, ir, upy), mx, my, both(p.wa), both(p.wd), heq);
+  if (p.fields || p.uout) {
+    const f2 half = vset<f2>(0.5f), px = vfma(half, Fx, jx), py = vfma(half, Fy, jy);
+    if (p.fields) {
+      const f2 e = equilibrium_sum(heq, 1.0f);
+      float *a = p.fields + self, *b = a + NFIELD * P;
+      a[0] = lo(d);
+      a[P] = lo(px);
+      a[2 * P] = lo(py);
+      a[3 * P] = lo(e);
+      b[0] = hi(d);
+      b[P] = hi(px);
+      b[2 * P] = hi(py);
+      b[3 * P] = hi(e);
+    }
+    if (p.uout) {
+      // the solvent velocity of Eq. (4)
+      const float rs = lo(rho) + hi(rho);
+      p.uout[self] = (lo(px) + hi(px)) / rs;
+      p.uout[P + self] = (lo(py) + hi(py)) / rs;
+    }
+  }
+  // mass-exact collision (collide_store_me): the exact sum D of the pulled
+  // values less the exact sum S of the eight stored moving populations
+  f2 Dh = h[0], Dl = vset<f2>(0.f), Sh, Sl = vset<f2>(0.f);
+#pragma unroll
+  for (int i = 1; i < 9; i++) {
+    f2 s, e;
+    two_sum(Dh, h[i], s, e);
+    Dh = s;
+    Dl = vadd(Dl, e);
+  }
+  S *f0 = (S *)p.fout, *f1 = f0 + 9 * P;
+#pragma unroll
+  for (int i = 1; i < 9; i++) {
+    f2 v = vfma(om, vsub(heq[i], h[i]), h[i]);
+    if constexpr (sizeof(S) == 4) {
+      f0[i * P + self] = lo(v);
+      f1[i * P + self] = hi(v);
+    } else {
+      // 16-bit dither: an independent hash per store
+      const uint32_t r0 = p.sr_seed ? (rnd(p.sr_seed, hself, 0, i) | 1u) : 0u;
+      const uint32_t r1 = p.sr_seed ? (rnd(p.sr_seed, hself, 1, i) | 1u) : 0u;
+      v = mk2(Store<S>::st_ret(f0, i * P + self, lo(v), p.scale, p.inv_scale, r0),
+              Store<S>::st_ret(f1, i * P + self, hi(v), p.scale, p.inv_scale, r1));
+    }
+    if (i == 1) {
+      Sh = v;
+    } else {
+      f2 s, e;
+      two_sum(Sh, v, s, e);
+      Sh = s;
+      Sl = vadd(Sl, e);
+    }
+  }
+  f2 rh, rl, h0, rem;
+  two_sum(Dh, vsub(vset<f2>(0.f), Sh), rh, rl);
+  rl = vadd(rl, vsub(Dl, Sl));
+  two_sum(rh, rl, h0, rem);
+  Store<S>::st(f0, self, last_bit(lo(h0), lo(rem), rnd(p.step_seed, hself, 0, 9)), p.scale,
+               p.sr_seed ? (rnd(p.sr_seed, hself, 0, 0) | 1u) : 0u);
+  Store<S>::st(f1, self, last_bit(hi(h0), hi(rem), rnd(p.step_seed, hself, 1, 9)), p.scale,
+               p.sr_seed ? (rnd(p.sr_seed, hself, 1, 0) | 1u) : 0u);
+}
+
 // ---------------------------------------------------------------------
 // inlet/outlet rules in one rotated form.
 //
