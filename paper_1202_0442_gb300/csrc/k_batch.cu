@@ -54,11 +54,11 @@ __device__ __forceinline__ void batch_warp(const BatchLat &L, const S *fin, S *f
   else moments1<float, false, false>(h, L.rho_ref, 1.0f, n);
   n.Fx = vfma(n.rho, L.ax, L.fx);
   n.Fy = vfma(n.rho, L.ay, L.fy);
-  if (L.pm) shift1<float, true>(L.tau, n);
-  else shift1<float, false>(L.tau, n);
+  if (L.pm) shift1<float, true, sizeof(S) == 2>(L.tau, n);
+  else shift1<float, false, sizeof(S) == 2>(L.tau, n);
   float heq[9];
-  equilibrium1<float, false>(n, 1.0f, 1.0f / 9.0f, 1.0f / 36.0f, heq);
-  relax(h, heq, L.omega, 1.0f - L.omega);
+  equilibrium1<float, false, sizeof(S) == 2>(n, 1.0f, 1.0f / 9.0f, 1.0f / 36.0f, heq);
+  relax<sizeof(S) == 2 ? 2 : 0>(h, heq, L.omega, 1.0f - L.omega);
   if (L.sr) {
     // stochastic rounding as in the single-lattice kernels: one hash per
     // node and launch, a linear congruential step per pair of stores

@@ -167,7 +167,7 @@ __device__ __forceinline__ bool fluid_node(const FluidArgs &p, int x, int y, uin
     for (int c = 0; c < NC; c++)
       slip_fix<S>(p, c, (const S *)p.fin + (size_t)c * 9 * g.plane, x, y, bits, linv, h[c]);
   }
-  if (p.nopen) apply_openings<NC>(p, x, y, h, FOLD ? p.scale : 1.0f);
+  if (p.nopen) apply_openings<NC, sizeof(S) == 2>(p, x, y, h, FOLD ? p.scale : 1.0f);
   if constexpr (ME) {
     float F[NC][2];
 #pragma unroll
@@ -219,7 +219,7 @@ __device__ __forceinline__ void pull_two(const FluidArgs &p, int x, int y, uint3
 #pragma unroll
     for (int c = 0; c < 2; c++) {
       if (SLIP && (bits & DIAG_BITS)) slip_fix<S>(p, c, c ? b : a, x, y, bits, p.inv_scale, f[c]);
-      if (OPEN) apply_opening_c(p, c, x, y, f[c]);
+      if (OPEN) apply_opening_c<sizeof(S) == 2>(p, c, x, y, f[c]);
     }
 #pragma unroll
     for (int i = 0; i < 9; i++) h[i] = mk2(f[0][i], f[1][i]);
@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(SC_TX *SC_TY, 4) k_fluid_sc(const FluidArgs p)
       pull9<S>((const S *)p.fin + (size_t)c * 9 * g.plane, g, x, y, bits, p.inv_scale, h[c]);
       if (SLIP && (bits & DIAG_BITS))
         slip_fix<S>(p, c, (const S *)p.fin + (size_t)c * 9 * g.plane, x, y, bits, p.inv_scale, h[c]);
-      if (OPEN) apply_opening_c(p, c, x, y, h[c]);
+      if (OPEN) apply_opening_c<sizeof(S) == 2>(p, c, x, y, h[c]);
 #pragma unroll
       for (int i = 0; i < 9; i++) d += h[c][i];
     }
@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(SC_TX *SC_TY, 4) k_fluid_sc(const FluidArgs p)
         pull9<S>((const S *)p.fin + (size_t)c * 9 * g.plane, g, hx, hy, hb, p.inv_scale, hh);
         if (SLIP && (hb & DIAG_BITS))
           slip_fix<S>(p, c, (const S *)p.fin + (size_t)c * 9 * g.plane, hx, hy, hb, p.inv_scale, hh);
-        if (OPEN) apply_opening_c(p, c, hx, hy, hh);
+        if (OPEN) apply_opening_c<sizeof(S) == 2>(p, c, hx, hy, hh);
 #pragma unroll
         for (int i = 0; i < 9; i++) d += hh[i];
       }

@@ -148,7 +148,7 @@ __device__ __forceinline__ void gather(R m2, R m5, R m6, const R (&z)[9], R p4, 
 // strip.  Kept in shared memory (each lane reads its own), so that the loop
 // holds no registers for it.
 struct LaneOpen {
-  float m[2], b[2]; // its rule (rho u_n = m S + b), 0 where there is none
+  float m[2], b[2], r[2]; // its rule (rho u_n = m S + b), 0 where there is none
   int a0[2], a1[2]; // rows it spans
   int on;           // bit 0: node a has one, 1: node b; bits 2, 3: on xhi
   int rows;         // its rule depends on the row (bit 0: a, bit 1: b)
@@ -158,13 +158,13 @@ __device__ __forceinline__ void lane_open(const MarchLat &p, const MarchOpen &op
   int on = 0, rows = 0;
 #pragma unroll
   for (int j = 0; j < 2; j++) {
-    float m = 0.f, b = 0.f;
+    float m = 0.f, b = 0.f, r = 0.f;
     int a0 = 1, a1 = 0;
 #pragma unroll 1
     for (int k = 0; k < op.nopen; k++) {
       const int wall = span_wall(op.span[k]);
       if (x[j] != (wall == 0 ? 0 : p.nx - 1) || a0 <= a1) continue;
-      if (!opening_mb(op.span[k], op.rule[k], 0, 0, p.rho_ref, sc, m, b)) continue;
+      if (!opening_mb(op.span[k], op.rule[k], 0, 0, p.rho_ref, sc, m, b, r)) continue;
       a0 = op.span[k].wa0 >> 2;
       a1 = op.span[k].a1;
       on |= (1 | wall << 2) << j;
@@ -172,6 +172,7 @@ __device__ __forceinline__ void lane_open(const MarchLat &p, const MarchOpen &op
     }
     L.m[j] = m;
     L.b[j] = b;
+    L.r[j] = r;
     L.a0[j] = a0;
     L.a1[j] = a1;
   }
@@ -180,6 +181,7 @@ __device__ __forceinline__ void lane_open(const MarchLat &p, const MarchOpen &op
 }
 
 // the opening rules of the lane's nodes in row y
+template <bool S16>
 __device__ __forceinline__ void open_pair(const MarchLat &p, const MarchOpen &op, const LaneOpen &L, int y, float sc,
                                           f2 (&v)[9]) {
   const int in = L.on & ((y >= L.a0[0] && y <= L.a1[0] ? 5 : 0) | (y >= L.a0[1] && y <= L.a1[1] ? 10 : 0));
@@ -189,8 +191,8 @@ __device__ __forceinline__ void open_pair(const MarchLat &p, const MarchOpen &op
 #pragma unroll 1
     for (int k = 0; k < op.nopen; k++) {
       const int wall = span_wall(op.span[k]);
-      float mk = 0.f, bk = 0.f;
-      opening_mb(op.span[k], op.rule[k], 0, y, p.rho_ref, sc, mk, bk);
+      float mk = 0.f, bk = 0.f, rk;
+      opening_mb(op.span[k], op.rule[k], 0, y, p.rho_ref, sc, mk, bk, rk);
 #pragma unroll
       for (int j = 0; j < 2; j++)
         if ((L.rows >> j & 1) && (L.on >> (2 + j) & 1) == wall) {
@@ -202,8 +204,9 @@ __device__ __forceinline__ void open_pair(const MarchLat &p, const MarchOpen &op
     b = mk2(bb[0], bb[1]);
   }
   f2 l1, l5, l8, r3, r6, r7;
-  zou_he<0>(v, m, b, l1, l5, l8);
-  zou_he<1>(v, m, b, r3, r6, r7);
+  const f2 rho = mk2(L.r[0], L.r[1]);
+  zou_he<0, S16>(v, m, b, rho, l1, l5, l8);
+  zou_he<1, S16>(v, m, b, rho, r3, r6, r7);
   const bool la = (in & 5) == 1, lb = (in & 10) == 2, ra = (in & 5) == 5, rb = (in & 10) == 10;
   v[1] = mk2(la ? lo(l1) : lo(v[1]), lb ? hi(l1) : hi(v[1]));
   v[5] = mk2(la ? lo(l5) : lo(v[5]), lb ? hi(l5) : hi(v[5]));
@@ -223,14 +226,14 @@ __device__ __forceinline__ void collide_pair(const MarchLat &p, const MarchOpen 
   f2 v[9];
 #pragma unroll
   for (int i = 0; i < 9; i++) v[i] = P::val(h[i]);
-  if (OPEN) open_pair(p, *op, L, y, FOLD ? p.scale : 1.0f, v);
+  if (OPEN) open_pair<sizeof(S) == 2>(p, *op, L, y, FOLD ? p.scale : 1.0f, v);
   Node1<f2> n;
   moments1<f2, PM, FOLD>(v, p.rho_ref, p.inv_scale, n);
   n.Fx = vfma(n.rho, vset<f2>(p.ax), vset<f2>(p.fx));
   n.Fy = vfma(n.rho, vset<f2>(p.ay), vset<f2>(p.fy));
-  shift1<f2, PM>(p.tau, n);
+  shift1<f2, PM, sizeof(S) == 2>(p.tau, n);
   f2 heq[9];
-  equilibrium1<f2, FOLD>(n, p.scale, p.wa, p.wd, heq);
+  equilibrium1<f2, FOLD, sizeof(S) == 2>(n, p.scale, p.wa, p.wd, heq);
   if (fields) {
     const f2 half = vset<f2>(0.5f);
     fields[0] = n.drho;
@@ -238,7 +241,7 @@ __device__ __forceinline__ void collide_pair(const MarchLat &p, const MarchOpen 
     fields[2] = vadd(n.jy, vfma(half, n.Fy, n.jyl));
     fields[3] = equilibrium_sum(heq, FOLD ? p.inv_scale : 1.0f);
   }
-  relax<RX>(v, heq, p.omega, p.keep);
+  relax<sizeof(S) == 2 ? 2 : RX>(v, heq, p.omega, p.keep);
   if constexpr (sizeof(S) == 4) {
 #pragma unroll
     for (int i = 0; i < 9; i++) o[i] = v[i];
@@ -456,7 +459,8 @@ int launch_march_r(const MarchArgs &a, dim3 grid, dim3 block, cudaStream_t s) {
 
 template <class S, int SR>
 int launch_march_t(const MarchArgs &a, dim3 grid, dim3 block, cudaStream_t s) {
-  return a.l.omega >= 1.0f ? launch_march_r<S, SR, 1>(a, grid, block, s) : launch_march_r<S, SR, 2>(a, grid, block, s);
+  if constexpr (sizeof(S) == 2) return launch_march_r<S, SR, 2>(a, grid, block, s);
+  else return a.l.omega >= 1.0f ? launch_march_r<S, SR, 1>(a, grid, block, s) : launch_march_r<S, SR, 2>(a, grid, block, s);
 }
 
 }  // namespace

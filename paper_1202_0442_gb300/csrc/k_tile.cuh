@@ -37,7 +37,7 @@ struct TilePair {
 };
 
 struct TileOpen {
-  float m[2], b[2];  // the opening rule of the two nodes
+  float m[2], b[2], r[2];  // the opening rule of the two nodes
 };
 
 // word of iteration t (as the host's step_word): the rounding dither's seed
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile(const TileArgs t) {
     q.flags = min(d, 255) << 4 | s << 16;
     if (t.op.nopen && (gx == 0 || gx == p.nx - 1)) {
       TileOpen o;
-      o.m[0] = o.m[1] = o.b[0] = o.b[1] = 0.f;
+      o.m[0] = o.m[1] = o.b[0] = o.b[1] = o.r[0] = o.r[1] = 0.f;
       const int row[2] = {ga, gb};
 #pragma unroll 1
       for (int j = 0; j < t.op.nopen; j++) {
@@ -129,7 +129,8 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile(const TileArgs t) {
 #pragma unroll
         for (int n = 0; n < 2; n++) {
           if (row[n] < (t.op.span[j].wa0 >> 2) || row[n] > t.op.span[j].a1) continue;
-          if (!opening_mb(t.op.span[j], t.op.rule[j], 0, row[n], p.rho_ref, sc, o.m[n], o.b[n])) continue;
+          if (!opening_mb(t.op.span[j], t.op.rule[j], 0, row[n], p.rho_ref, sc, o.m[n], o.b[n], o.r[n]))
+            continue;
           q.flags |= (wall + 1) | (4 << n);
         }
       }
@@ -177,16 +178,16 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile(const TileArgs t) {
       }
       if (q.flags & 3) {
         const TileOpen o = opens[k];
-        const f2 m = mk2(o.m[0], o.m[1]), b = mk2(o.b[0], o.b[1]);
+        const f2 m = mk2(o.m[0], o.m[1]), b = mk2(o.b[0], o.b[1]), rho = mk2(o.r[0], o.r[1]);
         const bool la = q.flags & 4, lb = q.flags & 8;
         f2 h1, h5, h8;
         if ((q.flags & 3) == 1) {
-          zou_he<0>(v, m, b, h1, h5, h8);
+          zou_he<0, sizeof(S) == 2>(v, m, b, rho, h1, h5, h8);
           v[1] = mk2(la ? lo(h1) : lo(v[1]), lb ? hi(h1) : hi(v[1]));
           v[5] = mk2(la ? lo(h5) : lo(v[5]), lb ? hi(h5) : hi(v[5]));
           v[8] = mk2(la ? lo(h8) : lo(v[8]), lb ? hi(h8) : hi(v[8]));
         } else {
-          zou_he<1>(v, m, b, h1, h5, h8);
+          zou_he<1, sizeof(S) == 2>(v, m, b, rho, h1, h5, h8);
           v[3] = mk2(la ? lo(h1) : lo(v[3]), lb ? hi(h1) : hi(v[3]));
           v[6] = mk2(la ? lo(h5) : lo(v[6]), lb ? hi(h5) : hi(v[6]));
           v[7] = mk2(la ? lo(h8) : lo(v[7]), lb ? hi(h8) : hi(v[7]));
@@ -196,10 +197,10 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile(const TileArgs t) {
       moments1<f2, PM, FOLD>(v, p.rho_ref, p.inv_scale, nd);
       nd.Fx = vfma(nd.rho, vset<f2>(p.ax), vset<f2>(p.fx));
       nd.Fy = vfma(nd.rho, vset<f2>(p.ay), vset<f2>(p.fy));
-      shift1<f2, PM>(p.tau, nd);
+      shift1<f2, PM, sizeof(S) == 2>(p.tau, nd);
       f2 heq[9];
-      equilibrium1<f2, FOLD>(nd, p.scale, p.wa, p.wd, heq);
-      relax(v, heq, p.omega, p.keep);
+      equilibrium1<f2, FOLD, sizeof(S) == 2>(nd, p.scale, p.wa, p.wd, heq);
+      relax<sizeof(S) == 2 ? 2 : 0>(v, heq, p.omega, p.keep);
       S a[9], b[9];
       round_pair<S, SR>(v, seed, q.selfa, q.selfb, a, b);
       if (n < T) {

@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(TT_THREADS, 3) k_fluid_tma(const FluidArgs p, 
                                                 : i * L::PLANE + cself - EY(i) * L::COLS - EX(i);
         h[0][i] = Store<S>::ld_smem(sb, off, linv);
       }
-      if (p.nopen) apply_openings<1>(p, x, y, h, FOLD ? p.scale : 1.0f);
+      if (p.nopen) apply_openings<1, sizeof(S) == 2>(p, x, y, h, FOLD ? p.scale : 1.0f);
       collide_store<S, false, FOLD, SR>(p, x, y, bits, h[0]);
     }
     if (kn < ntiles && tid < L::ROWS * L::MW) msk0[(s ^ 1) * L::ROWS * L::MW + tid] = mnext;

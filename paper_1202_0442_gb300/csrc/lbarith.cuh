@@ -70,6 +70,17 @@ __device__ __forceinline__ float vrcp(float a) {
 }
 __device__ __forceinline__ f2 vrcp(f2 a) { return mk2(vrcp(lo(a)), vrcp(hi(a))); }
 
+__device__ __forceinline__ float vrcp_rn(float a) { return __frcp_rn(a); }
+__device__ __forceinline__ f2 vrcp_rn(f2 a) { return mk2(__frcp_rn(lo(a)), __frcp_rn(hi(a))); }
+__device__ __forceinline__ float vdiv_rn(float a, float b) { return __fdiv_rn(a, b); }
+__device__ __forceinline__ f2 vdiv_rn(f2 a, f2 b) { return mk2(__fdiv_rn(lo(a), lo(b)), __fdiv_rn(hi(a), hi(b))); }
+// a rounded product that may feed a sum (a fused multiply-add with a zero,
+// which nothing fuses further)
+template <class V>
+__device__ __forceinline__ V vprod(V a, V b) {
+  return vfma(a, b, vset<V>(-0.0f));
+}
+
 // error-free sum: s + e == a + b exactly (Knuth)
 template <class V>
 __device__ __forceinline__ void two_sum(V a, V b, V &s, V &e) {
@@ -163,6 +174,36 @@ __device__ __forceinline__ void equilibrium(V drho, V ux, V uy, V mx, V my, V wa
   heq[0] = vfma(vset<V>(-2.0f), vadd(vadd(A1, A2), vadd(A5, A6)), drho);
 }
 
+// The same equilibrium in the operations that 16-bit storage keeps: its long
+// runs were validated with them, and there a single changed rounding moves
+// a dither's decision and with it, within some tens of iterations, the
+// whole noise pattern.  u is a rounded quotient, the quadratic terms are
+// formed from u and rho.
+template <class V>
+__device__ __forceinline__ void equilibrium_16(V drho, V rho, V ux, V uy, V mx, V my, V wa, V wd, V (&heq)[9]) {
+  const V q = vmul(rho, vfma(ux, ux, vmul(uy, uy)));
+  const V sp = vadd(ux, uy), sm = vsub(uy, ux);  // e5.u and e6.u
+  const V c12 = vset<V>(1.0f / 12.0f), n12 = vset<V>(-1.0f / 12.0f), half = vset<V>(0.5f);
+  const V n6 = vset<V>(-1.0f / 6.0f), n24 = vset<V>(-1.0f / 24.0f);
+  const V rh = vmul(half, rho), re = vmul(vset<V>(0.125f), rho);
+  const V A1 = vfma(q, n6, vfma(drho, wa, vmul(vmul(rh, ux), ux)));
+  const V A2 = vfma(q, n6, vfma(drho, wa, vmul(vmul(rh, uy), uy)));
+  const V A5 = vfma(q, n24, vfma(drho, wd, vmul(vmul(re, sp), sp)));
+  const V A6 = vfma(q, n24, vfma(drho, wd, vmul(vmul(re, sm), sm)));
+  const V B5 = vprod(vmul(rho, sp), c12), t6 = vmul(rho, sm);
+  const V B1 = vfma(t6, c12, vsub(vmul(half, mx), B5));
+  const V B2 = vfma(t6, n12, vsub(vmul(half, my), B5));
+  heq[1] = vadd(A1, B1);
+  heq[3] = vsub(A1, B1);
+  heq[2] = vadd(A2, B2);
+  heq[4] = vsub(A2, B2);
+  heq[5] = vadd(A5, B5);
+  heq[7] = vsub(A5, B5);
+  heq[6] = vfma(t6, c12, A6);
+  heq[8] = vfma(t6, n12, A6);
+  heq[0] = vfma(vset<V>(-2.0f), vadd(vadd(A1, A2), vadd(A5, A6)), drho);
+}
+
 // sum of the equilibrium deviations (Mass_eq of the thermo command); un:
 // stored units -> physical units
 template <class V>
@@ -203,7 +244,8 @@ __device__ __forceinline__ void moments1(const V (&h)[9], float rho_ref, float u
   n.rho = vadd(vset<V>(rho_ref), n.drho);
 }
 
-template <class V, bool PM>
+// S16: 16-bit storage
+template <class V, bool PM, bool S16>
 __device__ __forceinline__ void shift1(float tau, Node1<V> &n) {
   const V t = vset<V>(tau);
   if (PM) {
@@ -213,21 +255,31 @@ __device__ __forceinline__ void shift1(float tau, Node1<V> &n) {
     n.mx = vfma(t, n.Fx, n.jx);
     n.my = vfma(t, n.Fy, n.jy);
   }
-  const V ir = vrcp(n.rho);
-  n.ux = vmul(n.mx, ir);
-  n.uy = vmul(n.my, ir);
+  if (S16) {
+    const V ir = vrcp_rn(n.rho);
+    n.ux = vprod(n.mx, ir);
+    n.uy = vprod(n.my, ir);
+  } else {
+    const V ir = vrcp(n.rho);
+    n.ux = vmul(n.mx, ir);
+    n.uy = vmul(n.my, ir);
+  }
 }
 
 // h_eq of the node; FOLD: in stored units (it is linear in drho and rho u
 // at fixed u), sc = 2^s
-template <class V, bool FOLD>
+template <class V, bool FOLD, bool S16>
 __device__ __forceinline__ void equilibrium1(const Node1<V> &n, float sc, float wa, float wd, V (&heq)[9]) {
+  V d = n.drho, r = n.rho, mx = n.mx, my = n.my;
   if (FOLD) {
     const V s = vset<V>(sc);
-    equilibrium(vmul(n.drho, s), n.ux, n.uy, vmul(n.mx, s), vmul(n.my, s), vset<V>(wa), vset<V>(wd), heq);
-  } else {
-    equilibrium(n.drho, n.ux, n.uy, n.mx, n.my, vset<V>(wa), vset<V>(wd), heq);
+    d = vmul(d, s);
+    r = vmul(r, s);
+    mx = vmul(mx, s);
+    my = vmul(my, s);
   }
+  if (S16) equilibrium_16(d, r, n.ux, n.uy, mx, my, vset<V>(wa), vset<V>(wd), heq);
+  else equilibrium(d, n.ux, n.uy, mx, my, vset<V>(wa), vset<V>(wd), heq);
 }
 
 // BGK: h becomes (1 - omega) h + omega h_eq.  For omega >= 1 in that form
@@ -237,8 +289,9 @@ __device__ __forceinline__ void equilibrium1(const Node1<V> &n, float sc, float 
 // (f = 4 and 1) carries 3.5 times less momentum noise after 150 iterations,
 // and flows near equilibrium the same.  For omega < 1 as h + omega (h_eq - h):
 // the noise is the lower there (tau = 1.5, body force: by 1.3), and the
-// node's sums are kept although 1 - omega may be rounded.  RX: 0 decided
-// here, 1 omega >= 1, 2 omega < 1 (decided by the launch: both forms in one
+// node's sums are kept although 1 - omega may be rounded; 16-bit storage
+// always takes that form (equilibrium_16).  RX: 0 decided here, 1 the first
+// form, 2 the second (decided by the launch: both forms in one
 // kernel cost the 32-register streaming kernel 12 bytes of spills and 1.5 %
 // at 1024^2).
 template <int RX = 0, class V>

@@ -46,11 +46,11 @@ __device__ __forceinline__ void collide_store(const FluidArgs &p, int x, int y, 
     n.Fx -= p.Gads[0] * psi * sx;
     n.Fy -= p.Gads[0] * psi * sy;
   }
-  shift1<float, PM>(p.tau[0], n);
+  shift1<float, PM, sizeof(S) == 2>(p.tau[0], n);
   S *out = (S *)p.fout;
   float heq[9];
-  equilibrium1<float, FOLD>(n, p.scale, p.wa[0], p.wd[0], heq);
-  relax<RX>(h, heq, p.omega[0], p.keep);
+  equilibrium1<float, FOLD, sizeof(S) == 2>(n, p.scale, p.wa[0], p.wd[0], heq);
+  relax<sizeof(S) == 2 ? 2 : RX>(h, heq, p.omega[0], p.keep);
   const float sc = FOLD ? 1.0f : p.scale;
   if (SR == 2) {
     // stochastic rounding: one hash per node, then a linear congruential
@@ -384,7 +384,9 @@ __device__ __forceinline__ void collide_store_two(const FluidArgs &p, int x, int
 // which is the set of printed rules for each wall and style (inlet: u_n =
 // +v, outlet: u_n = -v), written for deviations h = f - w rho_ref.  Either
 // way a = m S + b with m and b fixed by the opening (and, for a Poiseuille
-// profile, the node's place along it).
+// profile, the node's place along it).  16-bit storage forms the dirichlet
+// a as rho u_n by the quotient (equilibrium_16 says why): r is then the
+// density held, else 0.
 // ---------------------------------------------------------------------
 template <int WALL> __device__ __forceinline__ constexpr int PERM(int k) {
   // xlo: n=+x t=+y; xhi: n=-x t=+y; ylo: n=+y t=+x; yhi: n=-y t=-x
@@ -394,36 +396,43 @@ template <int WALL> __device__ __forceinline__ constexpr int PERM(int k) {
                    : (k == 1 ? 4 : k == 2 ? 3 : k == 3 ? 2 : k == 4 ? 1 : k == 5 ? 7 : k == 7 ? 5 : k);
 }
 
-template <int WALL, class V>
-__device__ __forceinline__ void zou_he(const V (&h)[9], V m, V b, V &h1, V &h5, V &h8) {
+__device__ __forceinline__ float hold(float a, float r) { return r != 0.f ? __fmul_rn(r, __fdiv_rn(a, r)) : a; }
+__device__ __forceinline__ f2 hold(f2 a, f2 r) { return mk2(hold(lo(a), lo(r)), hold(hi(a), hi(r))); }
+
+template <int WALL, bool S16, class V>
+__device__ __forceinline__ void zou_he(const V (&h)[9], V m, V b, V r, V &h1, V &h5, V &h8) {
   constexpr int c0 = PERM<WALL>(0), c2 = PERM<WALL>(2), c3 = PERM<WALL>(3), c4 = PERM<WALL>(4), c6 = PERM<WALL>(6),
                 c7 = PERM<WALL>(7);
   const V S = vfma(vset<V>(2.0f), vadd(vadd(h[c3], h[c6]), h[c7]), vadd(vadd(h[c0], h[c2]), h[c4]));
-  const V a = vfma(S, m, b), d = vsub(h[c2], h[c4]), sixth = vset<V>(1.0f / 6.0f);
+  V a = vfma(S, m, b);
+  if (S16) a = hold(a, r);
+  const V d = vsub(h[c2], h[c4]), sixth = vset<V>(1.0f / 6.0f);
   h1 = vfma(vset<V>(2.0f / 3.0f), a, h[c3]);
   h5 = vfma(sixth, a, vfma(vset<V>(-0.5f), d, h[c7]));
   h8 = vfma(sixth, a, vfma(vset<V>(0.5f), d, h[c6]));
 }
 
-template <int WALL>
-__device__ __forceinline__ void zou_he_node(float (&h)[9], float m, float b) {
+template <int WALL, bool S16>
+__device__ __forceinline__ void zou_he_node(float (&h)[9], float m, float b, float r) {
   float h1, h5, h8;
-  zou_he<WALL>(h, m, b, h1, h5, h8);
+  zou_he<WALL, S16>(h, m, b, r, h1, h5, h8);
   h[PERM<WALL>(1)] = h1;
   h[PERM<WALL>(5)] = h5;
   h[PERM<WALL>(8)] = h8;
 }
 
-// m and b of component c's rule at coordinate coord along the wall; false
+// m, b and r of component c's rule at coordinate coord along the wall; false
 // if the component has no velocity or density style there.  sc: the units
 // of h (the rule is homogeneous of degree one in h, drho and rho_ref, so
 // scaled storage units take sc = 2^s)
 __device__ __forceinline__ bool opening_mb(const OpenSpan &s, const OpenRule &r, int c, int coord, float rho_ref,
-                                           float sc, float &m, float &b) {
+                                           float sc, float &m, float &b, float &rho) {
   const int st = (r.bits >> (3 * c)) & 7;
+  rho = 0.f;
   if (st == OPEN_DIRICHLET) {
     m = -1.0f;
     b = vmul(r.val[c], sc);
+    rho = vadd(vmul(rho_ref, sc), b);
     return true;
   }
   if (st != OPEN_POISEUILLE && st != OPEN_UNIFORM) return false;
@@ -436,16 +445,17 @@ __device__ __forceinline__ bool opening_mb(const OpenSpan &s, const OpenRule &r,
 
 // apply the velocity/dirichlet rule r of the opening at s to component c's
 // h (in units sc)
+template <bool S16>
 __device__ __forceinline__ void apply_opening(const OpenSpan &s, const OpenRule &r, int c, float (&h)[9],
                                               int x, int y, float rho_ref, float sc = 1.0f) {
   const int wall = span_wall(s);
-  float m, b;
-  if (!opening_mb(s, r, c, wall <= 1 ? y : x, rho_ref, sc, m, b)) return;
+  float m, b, rho;
+  if (!opening_mb(s, r, c, wall <= 1 ? y : x, rho_ref, sc, m, b, rho)) return;
   switch (wall) {
-    case 0: zou_he_node<0>(h, m, b); break;
-    case 1: zou_he_node<1>(h, m, b); break;
-    case 2: zou_he_node<2>(h, m, b); break;
-    default: zou_he_node<3>(h, m, b); break;
+    case 0: zou_he_node<0, S16>(h, m, b, rho); break;
+    case 1: zou_he_node<1, S16>(h, m, b, rho); break;
+    case 2: zou_he_node<2, S16>(h, m, b, rho); break;
+    default: zou_he_node<3, S16>(h, m, b, rho); break;
   }
 }
 
@@ -453,6 +463,7 @@ __device__ __forceinline__ void apply_opening(const OpenSpan &s, const OpenRule 
 // rule of a component reads only that component's populations, so the
 // interforce kernel applies it per component, to its own node and to the
 // ring nodes whose densities it stages); h in unscaled units
+template <bool S16>
 __device__ __forceinline__ void apply_opening_c(const FluidArgs &p, int c, int x, int y, float (&h)[9]) {
   const Geometry &g = p.g;
   const int gy = grow(g, y);
@@ -460,12 +471,12 @@ __device__ __forceinline__ void apply_opening_c(const FluidArgs &p, int c, int x
 #pragma unroll 1
   for (int k = 0; k < p.nopen; k++) {
     if (!opening_has(p.span[k], x, gy, g.nx, g.gny)) continue;
-    apply_opening(p.span[k], p.rule[k], c, h, x, gy, p.rho_ref[c]);
+    apply_opening<S16>(p.span[k], p.rule[k], c, h, x, gy, p.rho_ref[c]);
     return;
   }
 }
 
-template <int NC>
+template <int NC, bool S16>
 __device__ __forceinline__ void apply_openings(const FluidArgs &p, int x, int y,
                                                float (&h)[NC][9], float sc = 1.0f) {
   const Geometry &g = p.g;
@@ -475,7 +486,7 @@ __device__ __forceinline__ void apply_openings(const FluidArgs &p, int x, int y,
   for (int k = 0; k < p.nopen; k++) {
     if (!opening_has(p.span[k], x, gy, g.nx, g.gny)) continue;
 #pragma unroll
-    for (int c = 0; c < NC; c++) apply_opening(p.span[k], p.rule[k], c, h[c], x, gy, p.rho_ref[c], sc);
+    for (int c = 0; c < NC; c++) apply_opening<S16>(p.span[k], p.rule[k], c, h[c], x, gy, p.rho_ref[c], sc);
     break;
   }
 }

@@ -148,7 +148,7 @@ struct MarchArgs {
 };
 
 // several iterations of a small lattice per launch (k_tile.cuh)
-constexpr int TILE_NODES = 2624;   // of a tile and its halo (230,912 B of shared memory)
+constexpr int TILE_NODES = 2512;   // of a tile and its halo (231,104 B of shared memory)
 constexpr int TILE_THREADS = 512;
 constexpr int TILE_STEPS = 12;     // most iterations per launch
 struct TileArgs {
