@@ -117,7 +117,8 @@ int build_tiles(lb_batch *b) {
 
 // the tasks of k_march_batch, if the batch suits it: one rounding and
 // momentum mode, strips that fill their lanes, and enough nodes (measured:
-// 24 lattices of 1.9 M nodes 1.5 times faster than one iteration per launch;
+// 24 lattices of 1.9 M nodes in FP16 1.3 times faster than one iteration per
+// launch, 6 lattices of 0.6 M in FP32 1.15, 4 of 0.3 M in FP32 0.95, in FP16 1.1;
 // below some 320 K nodes the few rows per warp are a serial chain, as in
 // march_ok)
 int build_march(lb_batch *b) {
@@ -127,7 +128,7 @@ int build_march(lb_batch *b) {
     nodes += (int64_t)c->nx * c->ny;
     slots += (int64_t)((c->nx + MARCH_COLS - 1) / MARCH_COLS) * 64 * c->ny;
   }
-  if (nodes < 320000 || nodes * 5 < slots * 3) return LB_OK;
+  if (nodes < (b->storage == ST_FP32 ? 450000 : 320000) || nodes * 5 < slots * 3) return LB_OK;
   int sms = 0;
   BCK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
   // rows per warp: two or more waves of 16 warps per SM, where that leaves 8
