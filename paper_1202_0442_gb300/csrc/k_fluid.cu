@@ -242,12 +242,30 @@ __device__ __forceinline__ void pull_two(const FluidArgs &p, int x, int y, uint3
 // barrier waits on fewer warps; the ring costs 33 % more pulls, from L1/L2)
 constexpr int SC_TX = 32, SC_TY = 8;
 
-template <class S, int NC, bool SLIP, bool OPEN>
+// expm1 of both halves: the Taylor series up to |a| = 0.35 (its first term
+// left out is below 2e-8 of the result there), else the library's
+__device__ __forceinline__ f2 expm1_two(f2 a) {
+  if (fmaxf(fabsf(lo(a)), fabsf(hi(a))) > 0.35f) return mk2(expm1f(lo(a)), expm1f(hi(a)));
+  const f2 one = vset<f2>(1.0f);
+  f2 s = vfma(a, vset<f2>(1.0f / 7.0f), one);
+  s = vfma(vmul(a, vset<f2>(1.0f / 6.0f)), s, one);
+  s = vfma(vmul(a, vset<f2>(1.0f / 5.0f)), s, one);
+  s = vfma(vmul(a, vset<f2>(1.0f / 4.0f)), s, one);
+  s = vfma(vmul(a, vset<f2>(1.0f / 3.0f)), s, one);
+  s = vfma(vmul(a, vset<f2>(0.5f)), s, one);
+  return vmul(a, s);
+}
+
+// One component.  The nodes' 1/rho is staged beside rho - rho_ref, so that a
+// neighbour's difference takes no division, and opposite neighbours share
+// packed operations (777 x 500 FP32, 10 iterations: 200 -> 176 us; eight
+// expm1f calls and eight divisions per node before).
+template <class S, bool SLIP, bool OPEN>
 __global__ void __launch_bounds__(SC_TX *SC_TY, 4) k_fluid_sc(const FluidArgs p) {
-  // rho - rho_ref of every component for the tile and a one-node ring; slot
+  // rho - rho_ref and 1/rho for the tile and a one-node ring; slot
   // (ty + 1, tx + 1) holds node (x0 + tx, y0 + ty) wrapped periodically.
   // Solid nodes are told apart by the mask bits, not by the stored value.
-  __shared__ float sd[NC][SC_TY + 2][SC_TX + 2];
+  __shared__ float2 sd[SC_TY + 2][SC_TX + 2];
   dep_wait();
   const Geometry &g = p.g;
   const int tx = threadIdx.x, ty = threadIdx.y;
@@ -259,20 +277,18 @@ __global__ void __launch_bounds__(SC_TX *SC_TY, 4) k_fluid_sc(const FluidArgs p)
   // the wrapped node's)
   const uint32_t bits = __ldg(p.nbc + (size_t)y * g.pitch + x);
   const bool solid = (bits >> 4) & 1u;
-  float h[NC][9];
-#pragma unroll
-  for (int c = 0; c < NC; c++) {
+  const S *fin = (const S *)p.fin;
+  float h[1][9];
+  auto density = [&](int xx, int yy, uint32_t b, float(&f)[9]) {
+    pull9<S>(fin, g, xx, yy, b, p.inv_scale, f);
+    if (SLIP && (b & DIAG_BITS)) slip_fix<S>(p, 0, fin, xx, yy, b, p.inv_scale, f);
+    if (OPEN) apply_opening_c<sizeof(S) == 2>(p, 0, xx, yy, f);
     float d = 0.f;
-    if (!solid) {
-      pull9<S>((const S *)p.fin + (size_t)c * 9 * g.plane, g, x, y, bits, p.inv_scale, h[c]);
-      if (SLIP && (bits & DIAG_BITS))
-        slip_fix<S>(p, c, (const S *)p.fin + (size_t)c * 9 * g.plane, x, y, bits, p.inv_scale, h[c]);
-      if (OPEN) apply_opening_c<sizeof(S) == 2>(p, c, x, y, h[c]);
 #pragma unroll
-      for (int i = 0; i < 9; i++) d += h[c][i];
-    }
-    sd[c][ty + 1][tx + 1] = d;
-  }
+    for (int i = 0; i < 9; i++) d += f[i];
+    return make_float2(d, 1.0f / (p.rho_ref[0] + d));
+  };
+  sd[ty + 1][tx + 1] = solid ? make_float2(0.f, 0.f) : density(x, y, bits, h[0]);
   // ring: 2 (TX + 2) + 2 TY slots, one thread each
   const int tid = ty * SC_TX + tx;
   constexpr int NRING = 2 * (SC_TX + 2) + 2 * SC_TY;
@@ -284,61 +300,35 @@ __global__ void __launch_bounds__(SC_TX *SC_TY, 4) k_fluid_sc(const FluidArgs p)
     else { sx = SC_TX + 1; sy = tid - 2 * (SC_TX + 2) - SC_TY + 1; }
     const int hx = wrapi(x0 + sx - 1, g.nx), hy = wrapi(y0 + sy - 1, g.ny);
     const uint32_t hb = __ldg(p.nbc + (size_t)hy * g.pitch + hx);
-    const bool hs = (hb >> 4) & 1u;
-#pragma unroll
-    for (int c = 0; c < NC; c++) {
-      float d = 0.f;
-      if (!hs) {
-        float hh[9];
-        pull9<S>((const S *)p.fin + (size_t)c * 9 * g.plane, g, hx, hy, hb, p.inv_scale, hh);
-        if (SLIP && (hb & DIAG_BITS))
-          slip_fix<S>(p, c, (const S *)p.fin + (size_t)c * 9 * g.plane, hx, hy, hb, p.inv_scale, hh);
-        if (OPEN) apply_opening_c<sizeof(S) == 2>(p, c, hx, hy, hh);
-#pragma unroll
-        for (int i = 0; i < 9; i++) d += hh[i];
-      }
-      sd[c][sy][sx] = d;
-    }
+    float hh[9];
+    sd[sy][sx] = ((hb >> 4) & 1u) ? make_float2(0.f, 0.f) : density(hx, hy, hb, hh);
   }
   __syncthreads();
   if (!real || solid) return;
   // Since sum_i w_i e_i = 0, sum_i w_i psi(x + e_i) e_i equals
   // sum_i w_i (psi(x + e_i) - psi(x)) e_i; the differences are formed from
   // rho - rho_ref without cancellation:
-  //   two components: rho_n - rho_c = drho_n - drho_c (psi = rho)
-  //   one component:  psi_n - psi_c = psi_c expm1(rho0 (rho_n - rho_c)/(rho_n rho_c))
+  //   psi_n - psi_c = psi_c expm1(rho0 (rho_n - rho_c)/(rho_n rho_c))
   // and a solid neighbour contributes psi = 0, i.e. a difference -psi_c.
-  float F[NC][2];
   const int cx = tx + 1, cy = ty + 1;
+  const float2 me = sd[cy][cx];
+  const float psic = p.psi0 * expf(-p.sc_rho0 * me.y);
+  const f2 k = vset<f2>(p.sc_rho0 * me.y), dc = vset<f2>(me.x);
+  float F[1][2], t[4];
 #pragma unroll
-  for (int c = 0; c < NC; c++) {
-    const int o = (NC == 2) ? 1 - c : c;
-    const float dc = sd[o][cy][cx];
-    const float rc = p.rho_ref[o] + dc;
-    const float psic = (NC == 1) ? p.psi0 * expf(-p.sc_rho0 / rc) : rc;
-    float sx = 0.f, sy = 0.f;
-#pragma unroll
-    for (int i = 1; i < 9; i++) {
-      float diff;
-      if (nb(bits, i)) {
-        diff = -psic;
-      } else {
-        const float dn = sd[o][cy + EY(i)][cx + EX(i)];
-        if (NC == 1) {
-          const float rn = p.rho_ref[o] + dn;
-          diff = psic * expm1f(p.sc_rho0 * (dn - dc) / (rn * rc));
-        } else {
-          diff = dn - dc;
-        }
-      }
-      sx += W9(i) * (float)EX(i) * diff;
-      sy += W9(i) * (float)EY(i) * diff;
-    }
-    const float self = (NC == 1) ? psic : p.rho_ref[c] + sd[c][cy][cx];
-    F[c][0] = -p.G * self * sx;
-    F[c][1] = -p.G * self * sy;
+  for (int j = 0; j < 4; j++) {
+    // directions 1, 2, 5, 6 and their opposites
+    const int i = j < 2 ? j + 1 : j + 3;
+    const float2 a = sd[cy + EY(i)][cx + EX(i)], b = sd[cy - EY(i)][cx - EX(i)];
+    const f2 e = expm1_two(vmul(vmul(k, vsub(mk2(a.x, b.x), dc)), mk2(a.y, b.y)));
+    t[j] = (nb(bits, i) ? -1.0f : lo(e)) - (nb(bits, OPP(i)) ? -1.0f : hi(e));
   }
-  collide_store_me<S, NC>(p, x, y, bits, h, F);
+  // t: the difference of either direction's psi, over psi_c
+  const float sx = W9(1) * t[0] + W9(5) * (t[2] - t[3]), sy = W9(1) * t[1] + W9(5) * (t[2] + t[3]);
+  const float f = -p.G * psic * psic;
+  F[0][0] = f * sx;
+  F[0][1] = f * sy;
+  collide_store_me<S, 1>(p, x, y, bits, h, F);
 }
 
 // k_fluid_sc for two components, both in every packed operation: one index
@@ -477,10 +467,10 @@ int launch_fluid_t(int nc, bool sc, bool me, const FluidArgs &a, cudaStream_t s)
     // kernel without openings registers (spills in the two-component one)
     const bool op = a.nopen > 0;
     if (a.slip) {
-      if (nc == 1) launch_pdl(op ? k_fluid_sc<S, 1, true, true> : k_fluid_sc<S, 1, true, false>, grd, blk, 0, s, a);
+      if (nc == 1) launch_pdl(op ? k_fluid_sc<S, true, true> : k_fluid_sc<S, true, false>, grd, blk, 0, s, a);
       else launch_pdl(op ? k_fluid_sc2<S, true, true> : k_fluid_sc2<S, true, false>, grd, blk, 0, s, a);
     } else {
-      if (nc == 1) launch_pdl(op ? k_fluid_sc<S, 1, false, true> : k_fluid_sc<S, 1, false, false>, grd, blk, 0, s, a);
+      if (nc == 1) launch_pdl(op ? k_fluid_sc<S, false, true> : k_fluid_sc<S, false, false>, grd, blk, 0, s, a);
       else launch_pdl(op ? k_fluid_sc2<S, false, true> : k_fluid_sc2<S, false, false>, grd, blk, 0, s, a);
     }
   } else {
