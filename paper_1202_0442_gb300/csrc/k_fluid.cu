@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(32 * LOC_BY, ((NC == 1 && !ME && !PM) ? (SLIP 
 // solvent velocity of this iteration, which stays in registers, and the
 // previous iteration's solute populations around it.
 template <class S, int SR, int Q, bool SLIP>
-__global__ void __launch_bounds__(32 * LOC_BY, 4 * 8 / LOC_BY) k_fluid_solute(const FluidArgs p, const SoluteArgs sp) {
+__global__ void __launch_bounds__(32 * LOC_BY, 5) k_fluid_solute(const FluidArgs p, const SoluteArgs sp) {
   dep_wait();
   const int x = blockIdx.x * 32 + threadIdx.x;
   const int y = p.g.clo + blockIdx.y * LOC_BY + threadIdx.y;

@@ -97,23 +97,28 @@ __device__ __forceinline__ uint32_t growth_bits(const GrowthArgs &a, int x, int 
 // deposit and the share slot of every neighbour, whether or not that
 // neighbour is fluid (the slots of solid neighbours are read and dropped),
 // so that one memory latency, not two, precedes the arithmetic.
+// waited: the shares (this step's, by the kernel before) may be read; else
+// they are waited for after the other loads are issued.  Returns 1 if the
+// node listed a pick.
 template <int Q>
-__device__ __forceinline__ void gather_grow_node(const GrowthArgs &a, int x, int y) {
+__device__ __forceinline__ int gather_grow_node(const GrowthArgs &a, int x, int y, bool waited = true) {
   const Geometry &g = a.g;
   const int xm = x ? x - 1 : g.nx - 1, xp = (x + 1 == g.nx) ? 0 : x + 1;
   const int ym = y ? y - 1 : g.ny - 1, yp = (y + 1 == g.ny) ? 0 : y + 1;
   const size_t self = (size_t)y * g.pitch + x;
   const uint32_t bits = growth_bits(a, x, y);
+  double b = a.b[self];
+  if (!waited) dep_wait();
   constexpr int I0 = Q == 4 ? 0 : 1;
   float slot[Q];
 #pragma unroll
   for (int i = I0; i < Q; i++) {
     const int ex = Q == 4 ? EX4(i) : EX(i), ey = Q == 4 ? EY4(i) : EY(i);
     const int xf = ex > 0 ? xp : (ex < 0 ? xm : x), yf = ey > 0 ? yp : (ey < 0 ? ym : y);
-    slot[i] = __ldg(a.db + (size_t)yf * g.pitch + xf);
+    slot[i] = __ldcg(a.db + (size_t)yf * g.pitch + xf);
   }
-  double b = a.b[self];
-  if (!((bits >> 4) & 1u) || (bits | (1u << 4)) == 0x1ffu) return;
+  int listed = 0;
+  if (!((bits >> 4) & 1u) || (bits | (1u << 4)) == 0x1ffu) return 0;
   // the fluid neighbours' shares, added in index order (FP64)
   double acc = 0.0;
 #pragma unroll
@@ -150,11 +155,15 @@ __device__ __forceinline__ void gather_grow_node(const GrowthArgs &a, int x, int
       const uint64_t key = a.seed ^ ((uint64_t)a.t * (uint64_t)g.nx * (uint64_t)g.gny + node);
       const int pick = (int)(splitmix64(key) % (uint64_t)n);
       const unsigned int off = pick == 0 ? c0 : pick == 1 ? c1 : pick == 2 ? c2 : c3;
-      if (off != 0xffffffffu && atomicExch(a.flip + off, 1u) == 0u) a.flist[atomicAdd(a.fcount, 1u)] = off;
+      if (off != 0xffffffffu && atomicExch(a.flip + off, 1u) == 0u) {
+        a.flist[atomicAdd(a.fcount, 1u)] = off;
+        listed = 1;
+      }
       b = 0.0;
     }
   }
   a.b[self] = b;
+  return listed;
 }
 
 // every solid node with a fluid neighbour in the rows [rlo, rhi)
@@ -185,21 +194,42 @@ __global__ void __launch_bounds__(256) k_surface_list(const GrowthArgs a) {
     a.slist[atomicAdd(a.scount, 1u)] = (unsigned int)((size_t)y * g.pitch + x);
 }
 
-// One CTA's part of a growth step: it turns the listed nodes solid (mask
-// bit, b = b0, their fluid and solute mass booked as removed, their
-// populations cleared), appends them to the surface list if there is one,
-// refreshes the neighbour codes around them, then empties the list (the
-// entries stay, their number moves to fcount[1] for the host to read).
+// One CTA's part of a growth step: it turns the n listed nodes solid (mask
+// bit, the bit of the node in the neighbour codes around it, b = b0, their
+// fluid and solute mass booked as removed, their populations cleared),
+// appends them to the surface list if there is one, then empties the list
+// (the entries stay, their number moves to fcount[1] for the host to read).
 // Flips of one step are independent of each other, so their order does not
-// matter.  The list and its count are read from L2: other CTAs of the same
-// kernel may have written them.
+// matter.  The list is read from L2: other CTAs of the same kernel may have
+// written it.  After the list entry everything is issued at once: the codes
+// by atomic ORs that wait for nothing (recomputing them from the mask took a
+// barrier and two more dependent loads), the booked masses' loads beside the
+// populations'.
 template <class S>
 __device__ __forceinline__ void apply_flips_cta(const GrowthArgs &a) {
   const Geometry &g = a.g;
+  // the thread's first entry is loaded beside the count (the list has room
+  // for every node slot)
+  unsigned int first = threadIdx.x / 10u < (unsigned int)g.plane ? __ldcg(a.flist + threadIdx.x / 10u) : 0u;
   const unsigned int n = __ldcg(a.fcount);
-  for (unsigned int k = threadIdx.x; k < n; k += blockDim.x) {
-    const size_t self = __ldcg(a.flist + k);
+  for (unsigned int k = threadIdx.x; k < 10u * n; k += blockDim.x) {
+    const unsigned int e = k / 10u;
+    const int d = (int)(k - 10u * e);
+    const size_t self = k == threadIdx.x ? first : __ldcg(a.flist + e);
     const int y = (int)(self / (size_t)g.pitch), x = (int)(self - (size_t)y * g.pitch);
+    if (d < 9) {
+      // node (x, y) is neighbour (-dx, -dy) of node (x + dx, y + dy)
+      const int dx = d % 3 - 1, dy = d / 3 - 1;
+      int xn = x + dx, yn = y + dy;
+      xn = xn < 0 ? g.nx - 1 : (xn == g.nx ? 0 : xn);
+      yn = yn < 0 ? g.ny - 1 : (yn == g.ny ? 0 : yn);
+      const size_t c = (size_t)yn * g.pitch + xn;
+      atomicOr(reinterpret_cast<unsigned int *>(a.nbc) + (c >> 1), (1u << NBPOS(-dx, -dy)) << (16 * (c & 1)));
+      continue;
+    }
+    double rem[3] = {0.0, 0.0, 0.0};
+    for (int c = 0; c < a.nc; c++) rem[c] = a.removed[(size_t)c * g.plane + self];
+    if (a.gpop) rem[2] = a.removed[(size_t)a.nc * g.plane + self];
     a.flip[self] = 0u;
     atomicOr(a.mask + (size_t)y * g.mw + (x >> 5), 1u << (x & 31));
     if (a.slist) a.slist[atomicAdd(a.scount, 1u)] = (unsigned int)self;
@@ -209,7 +239,7 @@ __device__ __forceinline__ void apply_flips_cta(const GrowthArgs &a) {
       S *fp = (S *)a.f_prev + (size_t)c * 9 * g.plane;
       float d = 0.f;
       for (int i = 0; i < 9; i++) d += Store<S>::ld(f, (size_t)i * g.plane + self, a.inv_scale);
-      a.removed[(size_t)c * g.plane + self] += (double)a.rho_ref[c] + (double)d;
+      a.removed[(size_t)c * g.plane + self] = rem[c] + ((double)a.rho_ref[c] + (double)d);
       // a solid node holds no populations: its slots read zero in both
       // buffers, as the fluid kernels leave solid sectors untouched
       for (int i = 0; i < 9; i++) {
@@ -220,29 +250,8 @@ __device__ __forceinline__ void apply_flips_cta(const GrowthArgs &a) {
     if (a.gpop) {
       float m = 0.f;
       for (int i = 0; i < a.q; i++) m += a.gpop[(size_t)i * g.plane + self];
-      a.removed[(size_t)a.nc * g.plane + self] += (double)m;
+      a.removed[(size_t)a.nc * g.plane + self] = rem[2] + (double)m;
     }
-  }
-  __syncthreads();
-  // neighbour codes of the 3 x 3 neighbourhood of every flipped node, from
-  // the mask as it now stands (L2 reads: its words changed in this kernel).
-  // Overlapping neighbourhoods write the same value.
-  for (unsigned int k = threadIdx.x; k < 9u * n; k += blockDim.x) {
-    const size_t self = __ldcg(a.flist + k / 9);
-    const int y0 = (int)(self / (size_t)g.pitch), x0 = (int)(self - (size_t)y0 * g.pitch);
-    const int d = (int)(k % 9);
-    int x = x0 + d % 3 - 1, y = y0 + d / 3 - 1;
-    x = x < 0 ? g.nx - 1 : (x == g.nx ? 0 : x);
-    y = y < 0 ? g.ny - 1 : (y == g.ny ? 0 : y);
-    const int xs[3] = {x ? x - 1 : g.nx - 1, x, (x + 1 == g.nx) ? 0 : x + 1};
-    const int ys[3] = {y ? y - 1 : g.ny - 1, y, (y + 1 == g.ny) ? 0 : y + 1};
-    uint32_t b = 0;
-#pragma unroll
-    for (int j = 0; j < 3; j++)
-#pragma unroll
-      for (int i = 0; i < 3; i++)
-        b |= ((__ldcg(a.mask + (size_t)ys[j] * g.mw + (xs[i] >> 5)) >> (xs[i] & 31)) & 1u) << (j * 3 + i);
-    a.nbc[(size_t)y * g.pitch + x] = (uint16_t)b;
   }
   if (threadIdx.x == 0) {
     if (n) atomicAdd(a.nflips, (unsigned long long)n);
@@ -260,7 +269,10 @@ __device__ __forceinline__ void apply_flips_cta(const GrowthArgs &a) {
 // step's flips: one launch where the scan needs two.
 template <class S>
 __global__ void __launch_bounds__(256) k_grow_list(const GrowthArgs a) {
-  dep_wait();
+  // the list, the codes and the deposits are written by this kernel's own
+  // previous launch only, which completed before the kernel this one waits
+  // for began: read before the wait (a new list: after it)
+  if (a.fresh) dep_wait();
   const Geometry &g = a.g;
   const unsigned int stride = gridDim.x * blockDim.x;
   unsigned int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -268,22 +280,36 @@ __global__ void __launch_bounds__(256) k_grow_list(const GrowthArgs a) {
   // list has room for every node slot, so the slot exists)
   unsigned int self = k < (unsigned int)g.plane ? a.slist[k] : 0u;
   const unsigned int n = *a.scount;
-  const bool wrote = k < n;
+  bool waited = a.fresh;
+  int flips = 0;
   while (k < n) {
     const int y = (int)(self / (unsigned int)g.pitch), x = (int)(self - (unsigned int)y * (unsigned int)g.pitch);
-    if (a.q == 4) gather_grow_node<4>(a, x, y);
-    else gather_grow_node<9>(a, x, y);
+    flips += a.q == 4 ? gather_grow_node<4>(a, x, y, waited) : gather_grow_node<9>(a, x, y, waited);
+    waited = true;
     k += stride;
     if (k < n) self = a.slist[k];
   }
+  if (!waited) dep_wait();
+  // One ticket per CTA: its low half counts CTAs, its high half those that
+  // listed a node, so the last CTA knows without a load whether there are
+  // flips to apply (most steps have none).  The other CTAs' reads are
+  // complete when their ticket is drawn; what they wrote matters to the last
+  // one only where they listed a node, and only those fence.
   __shared__ unsigned int ticket;
-  if (wrote) __threadfence();
+  flips = __syncthreads_or(flips);
+  if (threadIdx.x == 0) {
+    const unsigned int mine = 1u + (flips ? 0x10000u : 0u);
+    if (flips) __threadfence();
+    ticket = atomicAdd(a.done, mine) + mine;
+  }
   __syncthreads();
-  if (threadIdx.x == 0) ticket = atomicAdd(a.done, 1u);
-  __syncthreads();
-  if (ticket != gridDim.x - 1) return;
-  __threadfence();
+  if ((ticket & 0xffffu) != gridDim.x) return;
   if (threadIdx.x == 0) *a.done = 0u;  // ready for the next step
+  if (!(ticket >> 16)) {
+    if (threadIdx.x == 0) a.fcount[1] = 0u;
+    return;
+  }
+  __threadfence();
   apply_flips_cta<S>(a);
 }
 

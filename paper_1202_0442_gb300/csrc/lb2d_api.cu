@@ -397,8 +397,7 @@ int commit(lb_ctx *ctx) {
   ctx->mask_host = m;
   ctx->mask_host_valid = true;
   if (ctx->slist) {
-    // blocks for the growth gather over the surface list: one entry per
-    // thread for the initial surface (the kernel strides over any more)
+    // the initial surface list's length
     size_t nsurf = 0;
     for (int y = 0; y < g.ny; y++)
       for (int x = 0; x < g.nx; x++) {
@@ -409,7 +408,7 @@ int commit(lb_ctx *ctx) {
             wet = !ctx->solid[(size_t)((y + dy + g.ny) % g.ny) * g.nx + (x + dx + g.nx) % g.nx];
         nsurf += wet;
       }
-    ctx->sblocks = (int)std::min<size_t>((nsurf + 255) / 256 + 1, (size_t)4 * ctx->sms);
+    ctx->nsurf = nsurf;
   }
 
   // hybrid boundary style: per-node reflection coefficients (0 on fluid
@@ -802,8 +801,15 @@ int one_step(lb_ctx *ctx, bool fields) {
       if (ctx->slist) {
         ga2.slist = ctx->slist;
         ga2.scount = ctx->scount;
-        ga2.sblocks = ctx->sblocks;
+        // one entry per thread for the list as far as the host knows it (its
+        // initial length and the flips of the last thermo record) and a
+        // quarter more; the kernel strides over any more, a chain of loads
+        // for each further entry (a run whose list had doubled: 2.5 us of
+        // the iteration's 9)
+        const size_t listed = ctx->nsurf + (ctx->thermo_valid ? (size_t)ctx->thermo.flips : 0);
+        ga2.sblocks = (int)std::min<size_t>((listed + listed / 4) / 256 + 2, (size_t)4 * ctx->sms);
         ga2.done = ctx->gdone;
+        ga2.fresh = ctx->slist_valid ? 0 : 1;
         if (!ctx->slist_valid) {
           CK(cudaMemsetAsync(ctx->scount, 0, sizeof(unsigned int), s));
           LAUNCH(launch_surface_list(ga2, s));

@@ -98,7 +98,7 @@ struct lb_ctx {
   // rebuilt at the next step whenever the device mask is replaced
   unsigned int *slist = nullptr, *scount = nullptr, *gdone = nullptr;
   bool slist_valid = false;
-  int sblocks = 0;
+  size_t nsurf = 0;  // the list's length when the device state was made
   uint16_t *nbc = nullptr;  // per-node neighbour codes of the streaming kernel
   // host copy of the device mask words while the two are known to agree
   // (lost once growth may have changed the device mask)

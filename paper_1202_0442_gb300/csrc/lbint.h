@@ -221,6 +221,7 @@ struct GrowthArgs {
                           // them; flipped nodes are appended), or nullptr:
                           // the rows [rlo, rhi) are scanned
   int sblocks;            // blocks of the launch over the list
+  int fresh;              // the list was built (or state uploaded) since the last launch over it
   unsigned int *done;     // CTAs of that launch finished (0 between launches)
   int q;
   int nopen;
