@@ -259,9 +259,10 @@ __device__ __forceinline__ f2 expm1_two(f2 a) {
 // One component.  The nodes' 1/rho is staged beside rho - rho_ref, so that a
 // neighbour's difference takes no division, and opposite neighbours share
 // packed operations (777 x 500 FP32, 10 iterations: 200 -> 176 us; eight
-// expm1f calls and eight divisions per node before).
+// expm1f calls and eight divisions per node before).  6 CTAs/SM at 40
+// registers without slip: 165 us (4 or 5: 176).
 template <class S, bool SLIP, bool OPEN>
-__global__ void __launch_bounds__(SC_TX *SC_TY, 4) k_fluid_sc(const FluidArgs p) {
+__global__ void __launch_bounds__(SC_TX *SC_TY, SLIP ? 4 : 6) k_fluid_sc(const FluidArgs p) {
   // rho - rho_ref and 1/rho for the tile and a one-node ring; slot
   // (ty + 1, tx + 1) holds node (x0 + tx, y0 + ty) wrapped periodically.
   // Solid nodes are told apart by the mask bits, not by the stored value.
