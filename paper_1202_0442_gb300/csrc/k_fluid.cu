@@ -532,8 +532,11 @@ int launch_march_bf16(const MarchArgs &a, dim3 grid, dim3 block, cudaStream_t s)
 int launch_march(int storage, MarchArgs &a, int sms, cudaStream_t s) {
   const MarchLat &g = a.l;
   a.sw = march_strip_width(g.nx);
-  const int all = (g.nx + a.sw - 1) / a.sw;
   const bool edges = a.op.nopen > 0;
+  // the strip before the last one advances the column after its own as well:
+  // with openings that must not be the last column of the lattice
+  while (edges && a.sw > 2 && g.nx % a.sw == 1) a.sw -= 2;
+  const int all = (g.nx + a.sw - 1) / a.sw;
   a.last = (all - 1) * a.sw;
   a.x0 = edges ? a.sw : 0;
   a.strips = edges ? std::max(all - 2, 0) : all;

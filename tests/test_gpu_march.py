@@ -2,7 +2,7 @@
 (lb_set_kernel "streaming"), bit for bit: populations, node fields, thermo
 records and the current buffer, at the widths and heights where its strips
 and segments end (one strip, odd widths whose last pair wraps, a lane's pair
-across the edge, a single row), with openings on the x walls, for every
+across the edge, a last strip of one column, a single row), with openings on the x walls, for every
 storage form.  An iteration count that is not a multiple of four leaves
 single iterations between the pairs and the record."""
 import numpy as np
@@ -52,7 +52,7 @@ def _workload(nx, ny, openings):
 
 @pytest.mark.parametrize("storage", list(STORAGE))
 @pytest.mark.parametrize("openings", [None, "dirichlet", "poiseuille"])
-@pytest.mark.parametrize("nx,ny", [(39, 8300), (121, 2700), (649, 501), (1025, 313), (320001, 1)])
+@pytest.mark.parametrize("nx,ny", [(39, 8300), (121, 2700), (649, 501), (1025, 313), (1741, 190), (3601, 90), (320001, 1)])
 def test_march_equals_single_iterations(nx, ny, openings, storage):
     if openings and ny < 8:
         pytest.skip("the openings' spans need a few rows")
