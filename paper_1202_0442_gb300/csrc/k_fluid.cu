@@ -12,7 +12,7 @@
 //   Eq. (3); surface_reaction, App. C) with the solvent velocity of Eq. (4)
 //   taken from registers: one pass for single-component runs with a solute
 //   and no intersolute.
-// k_fluid_sc: the same plus interforce, which needs the densities of the
+// k_fluid_sc, k_fluid_sc2 (two components): the same plus interforce, which needs the densities of the
 //   eight neighbours after this step's streaming and opening rules (the sums
 //   wrap periodically across every wall, openings or not).  Each CTA pulls
 //   the populations of its tile and of a one-node ring around it, applies
@@ -549,8 +549,9 @@ int launch_march(int storage, MarchArgs &a, int sms, cudaStream_t s) {
   // (16 warps of 128 registers per SM; shorter segments in more than one
   // wave repeat more rows at their ends: porous 1024^2 FP32 7.8 us per
   // iteration with one wave, 8.5 with one and a half or two).  The border
-  // strips take half as many (FP16 2003 x 1501: 23.2 us per iteration with
-  // as many rows, 21.1 with half, 21.8 with a third).
+  // strips take half as many (FP16 2003 x 1501, before 16-bit storage kept
+  // its longer arithmetic: 23.2 us per iteration with as many rows, 21.1 with
+  // half, 21.8 with a third).
   const int slots = sms * (16 / wpb);
   for (a.seg = 2;; a.seg++) {
     a.eseg = (a.seg + 1) / 2;

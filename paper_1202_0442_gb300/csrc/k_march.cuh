@@ -12,13 +12,14 @@
 // lanes and no barrier; all the arithmetic is packed, two nodes per
 // instruction.
 //
-// What bounds it: above L2 size the copy rate (porous 4096^2 FP32: 102 us
-// per iteration, 5.9 TB/s at 36 B per node and iteration; the one-iteration
+// What bounds it: above L2 size the copy rate (porous 4096^2 FP32: 105 us
+// per iteration, 5.8 TB/s at 36 B per node and iteration; the one-iteration
 // kernel takes 187); in L2 the latency of a row (16 warps of 128 registers
-// per SM): 1024^2 FP32 7.8 us against 10.2, FP16 2003 x 1501 21 against 32.
-// Tried on the way: the second iteration two rows behind, independent of
-// the first's row (168 registers, 12 warps): 1024^2 9.1 us; the rows' loop
-// unrolled once instead of twice (more register moves): 8.2.
+// per SM): 1024^2 FP32 7.8 us against 10.2; in 16-bit storage issue
+// (conversions, dithers, its longer arithmetic): FP16 2003 x 1501 25.5
+// against 32.4.  Tried on the way: the second iteration two rows behind,
+// independent of the first's row (168 registers, 12 warps): 1024^2 9.1 us;
+// the rows' loop not unrolled (more register moves): 8.2.
 #pragma once
 
 #include "lbbatch.h"
@@ -270,7 +271,8 @@ __device__ __forceinline__ void collide_pair(const MarchLat &p, const MarchOpen 
 // two iterations of rows [ys, ye) of the columns [X0, X1), by one
 // warp; OPEN: the strip's columns or their halo touch a wall with openings
 template <class S, bool PM, int SR, int RX, bool FIELDS, bool OPEN, int U>
-__device__ __forceinline__ void march_strip(const MarchLat &p, const MarchOpen *op, LaneOpen *lanes, int X0, int X1, int ys, int ye) {
+__device__ __forceinline__ void march_strip(const MarchLat &p, const MarchOpen *op, LaneOpen *lanes, int X0, int X1,
+                                            int ys, int ye) {
   using P = Pair<S>;
   using R = typename P::R;
   const int lane = threadIdx.x;
@@ -406,12 +408,12 @@ __global__ void __launch_bounds__(128, 4) k_march(const MarchArgs a) {
 }
 
 // the same for the lattices of a batch: a task per warp, the lattice's
-// parameters in shared memory (the loop not unrolled: with them in general
-// registers the copy spills 188 B instead of 60; 256 lattices FP32 192 us
-// per iteration against 200; k_batch takes 280, as does a launch per
-// iteration of this kernel's bytes, 72 B per node).  The launch numbers of its two iterations
-// are those of k_batch (tick), so the dithers do not depend on which of the
-// two kernels advances an iteration.
+// parameters in shared memory.  The loop is not unrolled: with them in
+// general registers the unrolled copy spills 188 B instead of 60 (256
+// lattices FP32 200 us per iteration against 192; k_batch, at 72 B per node
+// and iteration, takes 280).  The launch numbers of its two iterations are
+// those of k_batch (tick), so the dithers do not depend on which of the two
+// kernels advances an iteration.
 template <class S, bool PM, int SR>
 __global__ void __launch_bounds__(128, 4) k_march_batch(const MarchBatch b, int parity) {
   __shared__ MarchBatchLat lats[4];

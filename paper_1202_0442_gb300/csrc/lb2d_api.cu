@@ -7,7 +7,8 @@
 // state on the host, moves it to the GPU at the first call that needs
 // device memory, and then drives each iteration as a fixed sequence of
 // kernel launches on the caller's stream:
-//   fluid (k_fluid_local, k_fluid_sc or the fused k_fluid_solute) ->
+//   fluid (k_fluid_local, k_fluid_sc(2) or the fused k_fluid_solute; k_march
+//   or k_tile for several iterations at once) ->
 //   gradient openings -> solute -> growth (gather, decisions and flips) ->
 //   [thermo]
 // Slabs and their halo exchange are in lb2d_slab.cu, snapshots in
