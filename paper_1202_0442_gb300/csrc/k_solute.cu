@@ -82,9 +82,10 @@ __global__ void __launch_bounds__(256) k_solute(const SoluteArgs p) {
   solute_node<Q>(p, x, y, bits, __ldg(p.u + self), __ldg(p.u + g.plane + self));
 }
 
-// 3 x 3 solid neighbourhood of node (x, y) from its neighbour code
+// 3 x 3 solid neighbourhood of node (x, y) from its neighbour code, read
+// from L2: the growth step changes codes itself (k_grow_list says when)
 __device__ __forceinline__ uint32_t growth_bits(const GrowthArgs &a, int x, int y) {
-  return __ldg(a.nbc + (size_t)y * a.g.pitch + x);
+  return __ldcg(a.nbc + (size_t)y * a.g.pitch + x);
 }
 
 // Every solid node with a fluid neighbour adds the shares its fluid
@@ -107,7 +108,7 @@ __device__ __forceinline__ int gather_grow_node(const GrowthArgs &a, int x, int 
   const int ym = y ? y - 1 : g.ny - 1, yp = (y + 1 == g.ny) ? 0 : y + 1;
   const size_t self = (size_t)y * g.pitch + x;
   const uint32_t bits = growth_bits(a, x, y);
-  double b = a.b[self];
+  double b = __ldcg(a.b + self);
   if (!waited) dep_wait();
   constexpr int I0 = Q == 4 ? 0 : 1;
   float slot[Q];
@@ -269,17 +270,20 @@ __device__ __forceinline__ void apply_flips_cta(const GrowthArgs &a) {
 // step's flips: one launch where the scan needs two.
 template <class S>
 __global__ void __launch_bounds__(256) k_grow_list(const GrowthArgs a) {
-  // the list, the codes and the deposits are written by this kernel's own
-  // previous launch only, which completed before the kernel this one waits
-  // for began: read before the wait (a new list: after it)
+  // The list, the codes and the deposits are written by this kernel's own
+  // previous launch only.  The kernel this one waits for waited for that
+  // launch, and its blocks have all ended when this one's begin, so those
+  // writes are in L2 and are read before the wait (a new list: after it).
+  // Only from L2: no wait has dropped what this SM's L1 still holds of them,
+  // and a stale word of the list would be a wrong node.
   if (a.fresh) dep_wait();
   const Geometry &g = a.g;
   const unsigned int stride = gridDim.x * blockDim.x;
   unsigned int k = blockIdx.x * blockDim.x + threadIdx.x;
   // the thread's first entry is loaded beside the count, not after it (the
   // list has room for every node slot, so the slot exists)
-  unsigned int self = k < (unsigned int)g.plane ? a.slist[k] : 0u;
-  const unsigned int n = *a.scount;
+  unsigned int self = k < (unsigned int)g.plane ? __ldcg(a.slist + k) : 0u;
+  const unsigned int n = __ldcg(a.scount);
   bool waited = a.fresh;
   int flips = 0;
   while (k < n) {
@@ -287,7 +291,7 @@ __global__ void __launch_bounds__(256) k_grow_list(const GrowthArgs a) {
     flips += a.q == 4 ? gather_grow_node<4>(a, x, y, waited) : gather_grow_node<9>(a, x, y, waited);
     waited = true;
     k += stride;
-    if (k < n) self = a.slist[k];
+    if (k < n) self = __ldcg(a.slist + k);
   }
   if (!waited) dep_wait();
   // One ticket per CTA: its low half counts CTAs, its high half those that
