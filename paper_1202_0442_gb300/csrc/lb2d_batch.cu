@@ -377,6 +377,8 @@ int lb_batch_destroy(lb_batch *b) {
   if (b->d_tiles) cudaFree(b->d_tiles);
   if (b->d_counters) cudaFree(b->d_counters);
   if (b->d_tick) cudaFree(b->d_tick);
+  if (b->d_mlat) cudaFree(b->d_mlat);
+  if (b->d_mtasks) cudaFree(b->d_mtasks);
   delete b;
   return LB_OK;
 }
