@@ -46,6 +46,7 @@ sys.path.insert(0, ROOT)
 METRIC = "D2Q9 MLUPS and % of HBM roofline; 16-bit-storage & batched vs plain FP32 at ≤1e-5"
 WORKLOAD = "porous 1024x1024 (random discs r 8-24 seed 1, porosity 0.7, Zou-He rho 1.001/1.0, tau 0.8)"
 BYTES_PER_FLUID_NODE = {"fp32": 72, "fp16": 36, "bf16": 36}
+THERMO_EVERY = 100  # iterations between two thermo records of the timed run
 # measured against the FP64 oracle on this workload after its stated 10 000
 # iterations (tests/long_parity.py); the target for 16-bit storage is 2e-3
 ACCURACY_16 = {"fp16": "rel. u 7.3e-4 after 10 000 iterations: meets 2e-3",
@@ -590,8 +591,8 @@ def run_gb300(args, world, rank, local, dist):
     w = synth.porous()
     storage = args.storage
     lt = lb2d.from_workload(w, storage, h_max=2e-3, device=local, stream=stream.cuda_stream)
-    lt.thermo(100)
-    # the thermo record of every 100th step is copied to the host inside
+    lt.thermo(THERMO_EVERY)
+    # the thermo record of every THERMO_EVERY-th step is copied to the host inside
     # that step and read by the next thermo evaluation, so the host keeps
     # the stream fed
     lt.thermo_deferred(True)
@@ -629,13 +630,15 @@ def run_gb300(args, world, rank, local, dist):
     torch.cuda.synchronize()
     wall = time.perf_counter() - t_start
     launches = lt.launch_count() - launches0
-    last_thermo = lt.get_thermo()  # reads the last deferred record (raises on a non-finite sum)
+    # reads the last deferred record (raises on a non-finite sum), if the run
+    # has reached a thermo step
+    last_thermo = lt.get_thermo() if args.warmup + args.steps >= THERMO_EVERY else None
     if dist is not None:
         dist.barrier()
     clocks = sampler.stop() if sampler else None
     for k in range(args.steps):
         step_no = args.warmup + k + 1
-        thermo_step.append(step_no % 100 == 0)
+        thermo_step.append(step_no % THERMO_EVERY == 0)
     times = np.array([a.elapsed_time(b) for a, b in ev])
     ms_step = float(times.mean())
     plain = times[~np.array(thermo_step)] if (~np.array(thermo_step)).any() else times
@@ -727,9 +730,10 @@ def run_gb300(args, world, rank, local, dist):
         "config": {"workload": WORKLOAD, "nodes": nodes, "fluid_nodes": fluid,
                    "porosity": w.info["porosity"], "storage": storage,
                    "l2": "flushed before every timed step (write 2xL2, read 2xL2)",
-                   "thermo_every": 100,
+                   "thermo_every": THERMO_EVERY,
                    "thermo_records": "deferred: copied to the host inside the thermo step, read by the next "
-                                     f"thermo evaluation (the last, step {last_thermo['step']}, after the timed steps)",
+                                     f"thermo evaluation (the last, step {last_thermo['step']}, after the timed steps)"
+                                     if last_thermo else "none: fewer iterations than the thermo interval",
                    "parallelism": f"replicas x{world}"},
         "mflups": world * fluid / (ms_step * 1e-3) / 1e6,
         "bytes_all_nodes_frac": BYTES_PER_FLUID_NODE[storage] * nodes / (kernel_ms * 1e-3) / 1e9 / peaks()[0],
