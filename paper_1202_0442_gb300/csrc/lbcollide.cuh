@@ -291,18 +291,15 @@ __device__ __forceinline__ void collide_store_two(const FluidArgs &p, int x, int
     Fx = vfma(a, vset<f2>(sx), Fx);
     Fy = vfma(a, vset<f2>(sy), Fy);
   }
-  // common velocity sum(j/tau) / sum(rho/tau): quotients by a reciprocal and
-  // one correction
+  // common velocity sum(j/tau) / sum(rho/tau)
   const f2 nx = vmul(jx, om), ny = vmul(jy, om), nd = vmul(rho, om);
   const f2 num = mk2(lo(nx) + hi(nx), lo(ny) + hi(ny)), den = vset<f2>(lo(nd) + hi(nd));
-  const f2 rd = vset<f2>(vrcp(lo(den)));
-  const f2 q = vmul(num, rd);
-  const f2 up = vfma(vfma(vsub(vset<f2>(0.f), q), den, num), rd, q);
-  const f2 tx = vmul(tau, Fx), ty = vmul(tau, Fy), ir = vrcp(rho);
+  const f2 up = vdiv_rn(num, den);
+  const f2 tx = vmul(tau, Fx), ty = vmul(tau, Fy);
   const f2 upx = vset<f2>(lo(up)), upy = vset<f2>(hi(up));
   const f2 mx = vfma(rho, upx, tx), my = vfma(rho, upy, ty);
   f2 heq[9];
-  equilibrium(d, vfma(tx, ir, upx), vfma(ty, ir, upy), mx, my, both(p.wa), both(p.wd), heq);
+  equilibrium(d, vadd(upx, vdiv_rn(tx, rho)), vadd(upy, vdiv_rn(ty, rho)), mx, my, both(p.wa), both(p.wd), heq);
   if (p.fields || p.uout) {
     const f2 half = vset<f2>(0.5f), px = vfma(half, Fx, jx), py = vfma(half, Fy, jy);
     if (p.fields) {
