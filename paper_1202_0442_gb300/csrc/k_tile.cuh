@@ -158,12 +158,15 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile(const TileArgs t) {
       if (solid && n < T) continue;
       const int s = q.flags >> 16;
       f2 v[9];
+      // offsets of the lower node's sources in the row below it and of the
+      // upper node's in the row above it.  The region's first and last row
+      // have no such row; they are advanced with the other row of their pair
+      // only, their values used nowhere, and read the row next to it instead.
+      const int below = s < W ? W : 0, above = s >= (H - 2) * W ? 0 : W;
 #pragma unroll
       for (int i = 0; i < 9; i++) {
-        // sources of the lower and of the upper node; the pair's nodes that
-        // cannot be advanced yet or any more read inside the region, too
         const float *a = in + i * PS + s - EY(i) * W - EX(i);
-        v[i] = mk2(a[0], a[W]);
+        v[i] = mk2(a[EY(i) > 0 ? below : 0], a[EY(i) < 0 ? above : W]);
       }
       if (q.codes & NB) {
         const float *a = in + s;
