@@ -228,9 +228,8 @@ __device__ __forceinline__ void apply_flips_cta(const GrowthArgs &a) {
       atomicOr(reinterpret_cast<unsigned int *>(a.nbc) + (c >> 1), (1u << NBPOS(-dx, -dy)) << (16 * (c & 1)));
       continue;
     }
-    double rem[3] = {0.0, 0.0, 0.0};
-    for (int c = 0; c < a.nc; c++) rem[c] = a.removed[(size_t)c * g.plane + self];
-    if (a.gpop) rem[2] = a.removed[(size_t)a.nc * g.plane + self];
+    const double rem0 = a.removed[self], rem1 = a.nc > 1 ? a.removed[(size_t)g.plane + self] : 0.0;
+    const double remg = a.gpop ? a.removed[(size_t)a.nc * g.plane + self] : 0.0;
     a.flip[self] = 0u;
     atomicOr(a.mask + (size_t)y * g.mw + (x >> 5), 1u << (x & 31));
     if (a.slist) a.slist[atomicAdd(a.scount, 1u)] = (unsigned int)self;
@@ -240,7 +239,7 @@ __device__ __forceinline__ void apply_flips_cta(const GrowthArgs &a) {
       S *fp = (S *)a.f_prev + (size_t)c * 9 * g.plane;
       float d = 0.f;
       for (int i = 0; i < 9; i++) d += Store<S>::ld(f, (size_t)i * g.plane + self, a.inv_scale);
-      a.removed[(size_t)c * g.plane + self] = rem[c] + ((double)a.rho_ref[c] + (double)d);
+      a.removed[(size_t)c * g.plane + self] = (c ? rem1 : rem0) + ((double)a.rho_ref[c] + (double)d);
       // a solid node holds no populations: its slots read zero in both
       // buffers, as the fluid kernels leave solid sectors untouched
       for (int i = 0; i < 9; i++) {
@@ -251,7 +250,7 @@ __device__ __forceinline__ void apply_flips_cta(const GrowthArgs &a) {
     if (a.gpop) {
       float m = 0.f;
       for (int i = 0; i < a.q; i++) m += a.gpop[(size_t)i * g.plane + self];
-      a.removed[(size_t)a.nc * g.plane + self] = rem[2] + (double)m;
+      a.removed[(size_t)a.nc * g.plane + self] = remg + (double)m;
     }
   }
   if (threadIdx.x == 0) {
