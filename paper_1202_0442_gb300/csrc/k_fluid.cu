@@ -455,7 +455,8 @@ template <class S, int NC, bool ME, bool PM, int SR>
 void launch_local(const FluidArgs &a, cudaStream_t s) {
   dim3 blk(32, LOC_BY), grd((a.g.nx + 31) / 32, (a.g.chi - a.g.clo + LOC_BY - 1) / LOC_BY);
   if (a.slip) launch_pdl(k_fluid_local<S, NC, ME, PM, SR, true, 0>, grd, blk, 0, s, a);
-  else if constexpr (ME || PM) launch_pdl(k_fluid_local<S, NC, ME, PM, SR, false, 0>, grd, blk, 0, s, a);
+  else if constexpr (ME || PM || sizeof(S) == 2)  // one form of relax, or 16-bit storage's only one
+    launch_pdl(k_fluid_local<S, NC, ME, PM, SR, false, 0>, grd, blk, 0, s, a);
   else if (a.omega[0] >= 1.0f) launch_pdl(k_fluid_local<S, NC, ME, PM, SR, false, 1>, grd, blk, 0, s, a);
   else launch_pdl(k_fluid_local<S, NC, ME, PM, SR, false, 2>, grd, blk, 0, s, a);
 }
