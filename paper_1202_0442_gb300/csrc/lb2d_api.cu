@@ -1749,7 +1749,8 @@ int lb_iteration(lb_ctx *ctx, int Nt) {
   if (ctx->rank >= 0 && ctx->py > 1 && Nt > 1)
     return ctx->fail(LB_E_ORDER, "a slab of a lattice split into %d advances one iteration per call, its halo "
                      "rows exchanged between calls", ctx->py);
-  const bool several = several_ok(ctx), march = several && march_ok(ctx);
+  // (a call of one or two iterations has no use for either kernel)
+  const bool several = Nt > 2 && several_ok(ctx), march = several && march_ok(ctx);
   if (several && !march && !ctx->tile_steps) plan_tiles(ctx);
   for (int k = 0; k < Nt;) {
     // iterations up to the next one whose end the host looks at
