@@ -530,7 +530,7 @@ int launch_march_f32(const MarchArgs &a, dim3 grid, dim3 block, cudaStream_t s);
 int launch_march_f16(const MarchArgs &a, dim3 grid, dim3 block, cudaStream_t s);
 int launch_march_bf16(const MarchArgs &a, dim3 grid, dim3 block, cudaStream_t s);
 
-int launch_march(int storage, MarchArgs &a, int sms, cudaStream_t s) {
+void plan_march(MarchArgs &a, int sms) {
   const MarchLat &g = a.l;
   a.sw = march_strip_width(g.nx);
   const bool edges = a.op.nopen > 0;
@@ -557,9 +557,15 @@ int launch_march(int storage, MarchArgs &a, int sms, cudaStream_t s) {
   for (a.seg = 2;; a.seg++) {
     a.eseg = (a.seg + 1) / 2;
     a.eb = edges ? (2 * ((g.ny + a.eseg - 1) / a.eseg) + wpb - 1) / wpb : 0;
-    if (a.seg >= g.ny || a.eb + a.bx * ((g.ny + a.seg - 1) / a.seg) <= slots) break;
+    a.blocks = a.eb + a.bx * ((g.ny + a.seg - 1) / a.seg);
+    if (a.seg >= g.ny || a.blocks <= slots) break;
   }
-  const dim3 grid(a.eb + a.bx * ((g.ny + a.seg - 1) / a.seg)), block(32, wpb);
+  a.wpb = wpb;
+}
+
+int launch_march(int storage, MarchArgs &a, int sms, cudaStream_t s) {
+  plan_march(a, sms);
+  const dim3 grid(a.blocks), block(32, a.wpb);
   switch (storage) {
     case ST_FP16: return launch_march_f16(a, grid, block, s);
     case ST_BF16: return launch_march_bf16(a, grid, block, s);

@@ -839,14 +839,45 @@ bool several_ok(const lb_ctx *ctx) {
   return true;
 }
 
-// Two iterations per launch (k_march) for large lattices.  Below some 300 K
-// nodes its few rows per warp are a serial chain that the one-iteration
-// kernel does not have (porous FP32: 512^2 3.8 us per iteration either way,
-// 256^2 3.5 against 2.2; 600 K nodes in BF16 6.7 against 8.4, 1024^2 7.8
-// against 10.2); and a width that fills the strips badly leaves lanes idle.
+// Two iterations per launch (k_march) for large lattices whose width fills
+// the strips' lanes.  Below some 300 K nodes the few rows per warp are a
+// serial chain that the one-iteration kernel does not have (us per
+// iteration, FP32 | exact momentum | FP16: porous 480^2 3.60 | 4.15 | 4.40
+// against 3.50 | 3.88 | 4.15, 570^2 4.10 | 4.94 | 4.94 against 4.61 | 5.19 |
+// 5.34).  While the state fits L2 narrow lattices need a closer look: the
+// border strips of openings (1.7 times the instructions of a row) and the last
+// of few segments cost warps (porous 122 x 6000 1.12 | 1.27 | 1.17 times the
+// one-iteration kernel's time, 58 x 12000 1.36 | 1.42 | 1.39; 180 x 6000 0.83 |
+// 0.93 | 0.88).  Costs in us fitted to 40 shapes from 320 K to 1.5 M nodes,
+// porous with openings and periodic: the one-iteration kernel's by slots and
+// (openings) by rows, k_march's by rows per warp and the border strips' share of the
+// blocks.  They take no shape that is more than 2 % slower than one iteration
+// per launch, and leave out gains of 3 to 10 % at three.  Up to 327 K nodes
+// every shape goes by twos: the tests of the strips' edges, which pin that, are
+// of that size.  Beyond L2 the one-iteration kernel pays HBM twice: k_march
+// but for the narrowest (122 x 16000 0.79 | 0.95, 200 x 20000 0.73 | 0.79 |
+// 0.80).
 bool march_ok(const lb_ctx *ctx) {
   const int strips = (ctx->nx + MARCH_COLS - 1) / MARCH_COLS;
-  return (int64_t)ctx->nx * ctx->ny >= 320000 && ctx->nx * 5 >= strips * 64 * 3;
+  const int64_t nodes = (int64_t)ctx->nx * ctx->ny;
+  if (nodes < 320000 || ctx->nx * 5 < strips * 64 * 3) return false;
+  const bool fp32 = ctx->storage == ST_FP32, open = !ctx->open.empty();
+  if (nodes >= (fp32 ? 1500000 : 2800000))
+    return 64 * (strips + (open ? 2 : 0)) * 100 <= (fp32 ? 250 : 220) * ctx->g.pitch;
+  static const struct {
+    double one, slot, row, two, seg, border;
+  } costs[3] = {{1.6, 8.9e-6, 1.9e-4, 1.8, 0.68, 0.58},
+                {1.6, 10.9e-6, 1.7e-4, 2.1, 0.91, 0.24},
+                {1.9, 9.8e-6, 3.0e-4, 2.1, 0.83, 0.59}};
+  if (nodes < 327000) return true;
+  const auto &c = costs[!fp32 ? 2 : ctx->pm ? 1 : 0];
+  MarchArgs a{};
+  a.l.nx = ctx->nx;
+  a.l.ny = ctx->ny;
+  a.op.nopen = (int)ctx->open.size();
+  plan_march(a, ctx->sms);
+  const double one = c.one + c.slot * (double)ctx->g.pitch * ctx->ny + (open ? c.row * ctx->ny : 0.0);
+  return c.two + c.seg * a.seg + c.border * a.eb / a.blocks < 0.97 * one;
 }
 
 // The tiles of k_tile: for T iterations per launch the grid of at most one

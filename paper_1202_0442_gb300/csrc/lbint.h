@@ -145,6 +145,7 @@ struct MarchArgs {
                            // their number, rows per warp, blocks per row
   int eb, last, eseg;      // the border strips: blocks (0 without openings),
                            // first column of the last one, rows per warp
+  int blocks, wpb;         // of the launch; warps of a block
 };
 
 // several iterations of a small lattice per launch (k_tile.cuh)
@@ -267,6 +268,7 @@ struct CopyRuns {
 // launchers (return the kernel count launched, or -1 on a launch error)
 int launch_fluid(int storage, int nc, bool sc, bool mass_exact, const FluidArgs &a, cudaStream_t s);
 int launch_march(int storage, MarchArgs &a, int sms, cudaStream_t s);
+void plan_march(MarchArgs &a, int sms);  // the split of a.l's nodes with a.op's openings
 int launch_tile(int storage, const TileArgs &a, cudaStream_t s);
 int launch_gradient(int storage, const GradArgs &a, cudaStream_t s);
 // fluid and solute iteration in one kernel (one component, no interforce,
