@@ -116,11 +116,14 @@ int build_tiles(lb_batch *b) {
 }
 
 // the tasks of k_march_batch, if the batch suits it: one rounding and
-// momentum mode, strips that fill their lanes, and enough nodes (measured:
-// 24 lattices of 1.9 M nodes in FP16 1.3 times faster than one iteration per
-// launch, 6 lattices of 0.6 M in FP32 1.15, 4 of 0.3 M in FP32 0.95, in FP16 1.1;
-// below some 320 K nodes the few rows per warp are a serial chain, as in
-// march_ok)
+// momentum mode, and enough nodes in strips that fill their lanes (below, the few
+// rows per warp are a serial chain, as in march_ok).  Time over that of one
+// iteration per launch, FP32 | exact momentum | FP16.  Lanes filled to 0.75 or more:
+// 2 lattices of 480^2 (460 K) 1.06 | 1.08 | 0.85, 720^2 0.91 | 0.94 | 0.73, 22 of
+// 100 x 300 (660 K) 0.83 | 0.82 | 0.68, 24 uneven ones (2.2 M) 0.70 | 0.76 | 0.75.
+// Less: 40 of 128^2 (655 K) 1.10 | 1.20 | 1.00, 66 of 122^2 (982 K) 1.15 | 1.20 | 1.08, 80 of 128^2
+// (1.3 M) 0.99 | 1.12 | 0.95, 132 of 122^2 (2.0 M) 0.81 | 0.89 | 0.97; in 16 bits a
+// little more than one wave of warps (66 of 122^2: 1.3) is the only loss.
 int build_march(lb_batch *b) {
   int64_t nodes = 0, slots = 0;
   for (const lb_ctx *c : b->ctxs) {
@@ -128,7 +131,8 @@ int build_march(lb_batch *b) {
     nodes += (int64_t)c->nx * c->ny;
     slots += (int64_t)((c->nx + MARCH_COLS - 1) / MARCH_COLS) * 64 * c->ny;
   }
-  if (nodes < (b->storage == ST_FP32 ? 450000 : 320000) || nodes * 5 < slots * 3) return LB_OK;
+  const bool fp32 = b->storage == ST_FP32, full = nodes * 4 >= slots * 3;
+  if (nodes < (!fp32 ? 320000 : full ? 500000 : 1900000) || nodes * 5 < slots * 3) return LB_OK;
   int sms = 0;
   BCK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
   // rows per warp: two or more waves of 16 warps per SM, where that leaves 8
@@ -141,6 +145,7 @@ int build_march(lb_batch *b) {
     for (int y = 0; y < c->ny; y += seg)
       for (int x = 0; x < c->nx; x += sw) tasks.push_back(make_int4((int)k, x, y, seg));
   }
+  if (!full && (int)tasks.size() > 16 * sms && (int)tasks.size() * 2 < 3 * 16 * sms) return LB_OK;
   BCK(cudaMalloc((void **)&b->d_mlat, 2 * b->ctxs.size() * sizeof(MarchBatchLat)));
   BCK(cudaMalloc((void **)&b->d_mtasks, tasks.size() * sizeof(int4)));
   BCK(cudaMemcpyAsync(b->d_mtasks, tasks.data(), tasks.size() * sizeof(int4), cudaMemcpyHostToDevice, b->stream));

@@ -1,5 +1,6 @@
 """Which lattices go by two iterations per launch, told by the launch count:
-wide ones, and not the narrow ones with openings, which take longer that way."""
+wide ones, and not the narrow ones with openings or the batches of badly
+filled strips, which take longer that way."""
 import numpy as np
 import pytest
 
@@ -31,3 +32,13 @@ def test_lattice(nx, ny, pairs, storage):
     before = lt.launch_count()
     lt.iteration(8)
     assert lt.launch_count() - before == (4 if pairs else 8)
+
+
+@pytest.mark.parametrize("storage", ["fp32", "fp32_precise", "fp16_stochastic"])
+@pytest.mark.parametrize("count,nx,ny,pairs", [(66, 122, 122, False), (22, 100, 300, True)])
+def test_batch(count, nx, ny, pairs, storage):
+    st, kw = STORAGE[storage]
+    w = _workload(nx, ny, None)
+    b = lb2d.Batch([lb2d.from_workload(w, st, thermo=1 << 30, **kw) for _ in range(count)])
+    b.iteration(8, use_graph=False)
+    assert b.launch_count() == (4 if pairs else 8)
