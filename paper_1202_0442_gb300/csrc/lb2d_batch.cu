@@ -288,6 +288,17 @@ int batch_direct(lb_batch *b, int parity0, int n, bool march = true) {
   return rc;
 }
 
+// before launches that start with parity 0: after an odd number of launches
+// its work counter is cleared (the last launch, of parity 0 too, used it) and
+// takes up the launch number
+int batch_start(lb_batch *b) {
+  if (!b->odd) return LB_OK;
+  BCK(cudaMemsetAsync(b->d_counters, 0, sizeof(unsigned int), b->stream));
+  BCK(cudaMemcpyAsync(b->d_tick, b->d_tick + 1, sizeof(unsigned int), cudaMemcpyDeviceToDevice, b->stream));
+  b->odd = false;
+  return LB_OK;
+}
+
 void batch_advance(lb_batch *b, int n) {
   for (lb_ctx *c : b->ctxs) {
     c->cur = (c->cur + n) & 1;
@@ -403,13 +414,11 @@ int lb_batch_iteration(lb_batch *b, int Nt, int use_graph) {
   BCK(cudaSetDevice(b->device));
   int rc = sync_descs(b);
   if (rc != LB_OK) return rc;
-  if (b->odd && Nt > 0) {
-    // every call starts with parity 0: its work counter is cleared (the last
-    // launch, of parity 0 too, used it) and takes up the launch number
-    BCK(cudaMemsetAsync(b->d_counters, 0, sizeof(unsigned int), b->stream));
-    BCK(cudaMemcpyAsync(b->d_tick, b->d_tick + 1, sizeof(unsigned int), cudaMemcpyDeviceToDevice, b->stream));
+  if (Nt > 0) {
+    rc = batch_start(b);
+    if (rc != LB_OK) return rc;
+    b->odd = Nt & 1;
   }
-  if (Nt > 0) b->odd = Nt & 1;
   int done = 0;
   // poisoned members run without the graph (the poisoning is not captured)
   if (use_graph && !batch_poisoned(b)) {
@@ -470,6 +479,7 @@ int lb_batch_autotune(lb_batch *b, const char *cache_json) {
   }
   // keep the lattices' states: time on them, then put the states back
   int rc = sync_descs(b);
+  if (rc == LB_OK) rc = batch_start(b);
   if (rc != LB_OK) return rc;
   std::vector<void *> saved(b->ctxs.size(), nullptr);
   std::vector<size_t> sizes(b->ctxs.size());
