@@ -51,7 +51,7 @@ __device__ __forceinline__ void collide_store(const FluidArgs &p, int x, int y, 
   float heq[9];
   equilibrium1<float, FOLD, sizeof(S) == 2>(n, p.scale, p.wa[0], p.wd[0], heq);
   relax<sizeof(S) == 2 ? 2 : RX>(h, heq, p.omega[0], p.keep);
-  const float sc = FOLD ? 1.0f : p.scale;
+  // in stored units: FP16 is folded, the other types have no scale
   if (SR == 2) {
     // stochastic rounding: one hash per node, then a linear congruential
     // sequence, one step per pair of stores (each state is uniform for a
@@ -62,13 +62,13 @@ __device__ __forceinline__ void collide_store(const FluidArgs &p, int x, int y, 
 #pragma unroll
     for (int i = 0; i < 8; i += 2) {
       r = r * 1664525u + 1013904223u;
-      Store<S>::st2_dither(out, i * P + self, (i + 1) * P + self, vmul(h[i], sc), vmul(h[i + 1], sc), r);
+      Store<S>::st2_dither(out, i * P + self, (i + 1) * P + self, h[i], h[i + 1], r);
     }
     r = r * 1664525u + 1013904223u;
-    Store<S>::st_dither(out, 8 * P + self, vmul(h[8], sc), r);
+    Store<S>::st_dither(out, 8 * P + self, h[8], r);
   } else {
 #pragma unroll
-    for (int i = 0; i < 9; i++) Store<S>::st(out, i * P + self, h[i], sc);
+    for (int i = 0; i < 9; i++) Store<S>::st(out, i * P + self, h[i], 1.0f);
   }
   const float px = vadd(n.jx, vfma(0.5f, n.Fx, n.jxl)), py = vadd(n.jy, vfma(0.5f, n.Fy, n.jyl));
   if (p.fields) {
