@@ -542,8 +542,14 @@ int lb_get_flips(lb_ctx *ctx, int64_t *idx, int cap, int *count);
  * unbinds.  The library zeroes and writes it but never frees it; the caller
  * keeps it alive until lb_destroy.  A setup changed after binding
  * (storage, fluids, solute) is checked against the bound size when the
- * device state is created (first iteration or state upload: LB_E_ARG).  lb_current_buffer gives k such that f<k>
- * and g<k> hold the current state (it alternates every iteration). */
+ * device state is created (first iteration or state upload: LB_E_ARG).
+ * lb_current_buffer gives k such that f<k> and g<k> hold the current state:
+ * after a call of n iterations k has alternated n times.  The other buffer
+ * is working space and holds the state of an earlier iteration: the one
+ * before after a call of one iteration (and always where the library
+ * advances one iteration per launch), else one up to twelve iterations back,
+ * as a launch may advance several.  A program that needs the last two states
+ * calls lb_iteration(n - 1) and lb_iteration(1). */
 int lb_buffer_size(lb_ctx *ctx, const char *what, size_t *bytes);
 int lb_bind(lb_ctx *ctx, const char *what, void *dev, size_t bytes);
 int lb_current_buffer(lb_ctx *ctx, int *index);
@@ -616,14 +622,16 @@ int lb_lattice_info(lb_ctx *ctx, int *nx, int *ny, int *ncomp, int *q, int *px, 
 
 /* Group n committed single-component contexts of one device and stream
  * (periodic, no openings, no solute, same storage) so that lb_batch_iteration
- * advances all of them with one kernel launch per iteration.  The contexts
- * stay owned by the caller and must outlive the batch. */
+ * advances all of them with one kernel launch per iteration or per two.  The
+ * contexts stay owned by the caller and must outlive the batch. */
 int lb_batch_create(lb_ctx *const *ctxs, int n, lb_batch **out);
 int lb_batch_destroy(lb_batch *b);
 /* Advance every lattice of the batch Nt iterations; use_graph != 0
  * captures the launches in a CUDA graph and replays it. */
 int lb_batch_iteration(lb_batch *b, int Nt, int use_graph);
-/* Time the candidate tile shapes and work schedules and keep the fastest;
+/* Time the candidate tile shapes and work schedules of the launch that
+ * advances one iteration (batches that go by twos use it for the last one to
+ * three iterations of a call) and keep the fastest;
  * cache_json (may be NULL) is a file that stores the choice keyed by
  * device, shapes and storage. */
 int lb_batch_autotune(lb_batch *b, const char *cache_json);
