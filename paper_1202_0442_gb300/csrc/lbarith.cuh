@@ -82,7 +82,6 @@ __device__ __forceinline__ V vrcp(V a) {
 
 __device__ __forceinline__ float vrcp_rn(float a) { return __frcp_rn(a); }
 __device__ __forceinline__ f2 vrcp_rn(f2 a) { return mk2(__frcp_rn(lo(a)), __frcp_rn(hi(a))); }
-__device__ __forceinline__ float vdiv_rn(float a, float b) { return __fdiv_rn(a, b); }
 __device__ __forceinline__ f2 vdiv_rn(f2 a, f2 b) { return mk2(__fdiv_rn(lo(a), lo(b)), __fdiv_rn(hi(a), hi(b))); }
 // a rounded product that may feed a sum.  Of two nodes: one multiplication
 // each, which the compiler does not fuse with the packed sum (it does fuse a

@@ -4,8 +4,11 @@
     python profile_target.py shanchen2048 fp32
     python profile_target.py reactive fp32
     python profile_target.py batch256 fp32
+    python profile_target.py porous1024 fp32 8 streaming
+    python profile_target.py channel fp32 48
 
-Sets up the named workload on cuda:0, runs a fixed number of iterations
+Workload, storage, iterations and kernel (lb_set_kernel; "streaming": one
+iteration per launch where the default advances several).  Sets up the named workload on cuda:0, runs a fixed number of iterations
 (thermo off, so every launch is the same kernel sequence) and exits 0.
 Under ``ncu -k regex:<kernel> -s <skip> -c 1`` it gives one launch of that
 kernel on a lattice larger than L2 while keeping the device footprint to a
@@ -26,6 +29,8 @@ def main(argv=None) -> int:
     name = argv[0] if argv else "porous4096"
     storage = argv[1] if len(argv) > 1 else "fp32"
     iters = int(argv[2]) if len(argv) > 2 else 8
+    kernel = argv[3] if len(argv) > 3 else "auto"
+    import numpy as np
     import torch
 
     from paper_1202_0442_gb300 import build, lb2d, synth
@@ -35,6 +40,13 @@ def main(argv=None) -> int:
         w = synth.porous(4096, 4096, seed=1)
     elif name == "porous1024":
         w = synth.porous()
+    elif name == "channel":
+        w = synth.channel(64, 32, tau=1.0, gx=1e-6)
+    elif name == "vapour":
+        # one component with interforce, separating from a noisy density
+        w = synth.Workload(name="vapour", nx=777, ny=500, solid=np.zeros((500, 777), np.uint8),
+                           rho=[200.0 + np.random.default_rng(1).uniform(0.0, 1.0, (500, 777))],
+                           interforce=(-120.0, 4.0, 200.0), rho_ref=(200.0,))
     elif name == "shanchen2048":
         w = synth.shan_chen2(2048)
     elif name == "reactive":
@@ -54,7 +66,7 @@ def main(argv=None) -> int:
         return 0
     else:
         raise SystemExit(f"unknown workload {name}")
-    lt = lb2d.from_workload(w, storage, h_max=2e-3,
+    lt = lb2d.from_workload(w, storage, h_max=2e-3, kernel=kernel,
                             rounding="stochastic" if storage != "fp32" else "nearest")
     lt.thermo(1 << 30)
     lt.iteration(iters)
