@@ -125,7 +125,8 @@ constexpr uint32_t DIAG_BITS = (1u << NBPOS(-1, -1)) | (1u << NBPOS(1, -1)) | (1
 
 constexpr int LOC_BY = 8;
 
-// SR: 1 nearest, 2 stochastic (16-bit, not ME).  RX: the form of relax.  Scaled 16-bit storage without ME runs folded (collide_store).
+// SR: 1 nearest, 2 stochastic (16-bit, not ME).  RX: the form of relax.
+// Scaled 16-bit storage without ME runs folded (collide_store).
 // The update of node (x, y) given its neighbour code (called by every lane
 // of a warp: the warp votes on its solid lanes).  Returns false on solid
 // nodes and row padding.  uo, if given, receives the node's solvent
@@ -238,8 +239,8 @@ __device__ __forceinline__ void pull_two(const FluidArgs &p, int x, int y, uint3
   }
 }
 
-// 32 x 8 tiles, 4 CTAs/SM: measured fastest of 32 x {4, 8, 16, 32} (the
-// barrier waits on fewer warps; the ring costs 33 % more pulls, from L1/L2)
+// 32 x 8 tiles: measured fastest of 32 x {4, 8, 16, 32} (the barrier waits on
+// fewer warps; the ring costs 33 % more pulls, from L1/L2)
 constexpr int SC_TX = 32, SC_TY = 8;
 
 // expm1 of both halves: the Taylor series up to |a| = 0.35 (its first term
@@ -260,7 +261,11 @@ __device__ __forceinline__ f2 expm1_two(f2 a) {
 // neighbour's difference takes no division, and opposite neighbours share
 // packed operations (777 x 500 FP32, 10 iterations: 200 -> 176 us; eight
 // expm1f calls and eight divisions per node before).  6 CTAs/SM at 40
-// registers without slip: 165 us (4 or 5: 176).
+// registers without slip: 165 us (4 or 5: 176).  The force's error against
+// 64 bits (densities held exactly, 2-norm) is that of the divisions and
+// expm1f or less: densities 200 +- 0.5 1.61e-7 (1.62e-7), 200 +- 8 1.36e-7
+// (1.43e-7), 115 to 283 1.32e-7 (1.37e-7); a corrected quotient and a series
+// summed from its small end changed neither these nor the time.
 template <class S, bool SLIP, bool OPEN>
 __global__ void __launch_bounds__(SC_TX *SC_TY, SLIP ? 4 : 6) k_fluid_sc(const FluidArgs p) {
   // rho - rho_ref and 1/rho for the tile and a one-node ring; slot
@@ -336,9 +341,11 @@ __global__ void __launch_bounds__(SC_TX *SC_TY, SLIP ? 4 : 6) k_fluid_sc(const F
 // per population for both loads, one shared-memory word pair per neighbour,
 // and the collision of collide_store_two.  A solid node's staged density is
 // 0 (its deviation -rho_ref), so the force takes no test of the neighbours.
-// 64 registers without spills, as the scalar form had: 2048^2 FP32 154 us
-// per iteration against 175 (72 B per node and component: 89 at the copy
-// rate); still issue- and latency-bound at half the warps.  A warp per strip
+// 64 registers without spills, as the scalar form had (4 B with openings,
+// 48 to 64 B with slip: 1024^2 with slip 55 us per iteration against 60): 2048^2
+// FP32 154 us per iteration in a call of ten against 175, 144 in longer
+// ones (72 B per node and component: 89 at the copy rate); still issue- and
+// latency-bound at half the warps.  A warp per strip
 // that walks the rows (no ring, no barrier; 128 registers, 16 warps per SM)
 // took 195 to 260.
 template <class S, bool SLIP, bool OPEN>
@@ -548,11 +555,10 @@ void plan_march(MarchArgs &a, int sms) {
   a.bx = (a.strips + wpb - 1) / wpb;
   // Rows per warp: the fewest with which every block is resident at once
   // (16 warps of 128 registers per SM; shorter segments in more than one
-  // wave repeat more rows at their ends: porous 1024^2 FP32 7.8 us per
-  // iteration with one wave, 8.5 with one and a half or two).  The border
-  // strips take half as many (FP16 2003 x 1501, before 16-bit storage kept
-  // its longer arithmetic: 23.2 us per iteration with as many rows, 21.1 with
-  // half, 21.8 with a third).
+  // wave repeat more rows at their ends: porous 1024^2 FP32, with an earlier
+  // arithmetic, 7.8 us per iteration with one wave, 8.5 with one and a half or
+  // two).  The border strips take half as many (FP16 2003 x 1501, likewise:
+  // 23.2 us per iteration with as many rows, 21.1 with half, 21.8 with a third).
   const int slots = sms * (16 / wpb);
   for (a.seg = 2;; a.seg++) {
     a.eseg = (a.seg + 1) / 2;

@@ -12,14 +12,14 @@
 // lanes and no barrier; all the arithmetic is packed, two nodes per
 // instruction.
 //
-// What bounds it: above L2 size the copy rate (porous 4096^2 FP32: 105 us
-// per iteration, 5.8 TB/s at 36 B per node and iteration; the one-iteration
-// kernel takes 187); in L2 the latency of a row (16 warps of 128 registers
-// per SM): 1024^2 FP32 7.8 us against 10.2; in 16-bit storage issue
-// (conversions, dithers, its longer arithmetic): FP16 2003 x 1501 25.5
-// against 32.4.  Tried on the way: the second iteration two rows behind,
-// independent of the first's row (168 registers, 12 warps): 1024^2 9.1 us;
-// the rows' loop not unrolled (more register moves): 8.2.
+// What bounds it: above L2 size DRAM (porous 4096^2 FP32: 107 us per
+// iteration, 5.2 TB/s under ncu; the one-iteration kernel takes 196); in L2
+// the latency of a row (16 warps of 128 registers per SM): 1024^2 FP32 8.4 us
+// against 11.0; in 16-bit storage issue (conversions, dithers, its longer
+// arithmetic): FP16 2003 x 1501 24.4 against 33.7.  Tried on the way, with an earlier
+// arithmetic (1024^2 7.8 us): the second iteration two rows behind, independent of
+// the first's row (168 registers, 12 warps) 9.1 us; the rows' loop not
+// unrolled (more register moves) 8.2.
 #pragma once
 
 #include "lbbatch.h"
@@ -410,8 +410,9 @@ __global__ void __launch_bounds__(128, 4) k_march(const MarchArgs a) {
 // the same for the lattices of a batch: a task per warp, the lattice's
 // parameters in shared memory.  The loop is not unrolled: with them in
 // general registers the unrolled copy spills 188 B instead of 60 (256
-// lattices FP32 200 us per iteration against 192; k_batch, at 72 B per node
-// and iteration, takes 280).  The launch numbers of its two iterations are
+// lattices FP32, with an earlier arithmetic, 200 us per iteration against 192).
+// 256 lattices with exact momentum: 178 us per iteration, k_batch, at 72 B per
+// node and iteration, 270.  The launch numbers of its two iterations are
 // those of k_batch (tick), so the dithers do not depend on which of the two
 // kernels advances an iteration.
 template <class S, bool PM, int SR>

@@ -12,11 +12,12 @@
 // the other, per packed operation.
 //
 // What bounds it: the latency of an iteration (a pair's chain of loads,
-// packed arithmetic and stores, some 300 instructions, by 16 warps): 0.6 us
-// for the 64 x 32 channel, 1.1 for 256^2, besides 2 us and the loads of a
-// launch.  64 x 32, 100 iterations: 217 -> 110 us.  With 768 or 1024 threads
-// the lattices of one round gain nothing (64 x 32 0.84 and 1.08 us per
-// iteration against 0.83).
+// packed arithmetic and stores, some 300 instructions, by 16 warps): 0.7 us
+// for the 64 x 32 channel, 1.2 for 256^2, besides 2 us and the loads of a
+// launch.  Per iteration, against one per launch: 64 x 32 0.91 us against
+// 1.84, 256^2 1.75 against 2.35, 400^2 2.87 against 3.27.  With 768 or 1024 threads
+// the lattices of one round gain nothing (64 x 32, with an earlier arithmetic, 0.84
+// and 1.08 us per iteration against 0.83).
 #pragma once
 
 #include "lbcollide.cuh"

@@ -883,12 +883,16 @@ bool march_ok(const lb_ctx *ctx) {
 // The tiles of k_tile: for T iterations per launch the grid of at most one
 // block per SM whose tiles with their halo are the smallest, and the T that
 // costs the least per iteration, if that is less than the one-iteration
-// kernel's (T = 1).  Costs in us, from timings with T = 2..12: a launch 1.8 and
-// 3 per 1000 nodes read, an iteration 0.4 and 0.65 per round of the block's
-// threads over its pairs of nodes (porous FP32: 256^2 T = 5 1.73 per iteration,
-// T = 8 2.00, single 2.32; 400^2 T = 6 2.80, T = 3 3.78, single 3.09; 512^2
-// 3.90 against 3.83: not taken); the one-iteration kernel 1.75 and 8 per
-// million nodes.
+// kernel's (T = 1).  Costs in us, from FP32 timings with T = 2..12: a launch
+// 1.8 and 3 per 1000 nodes read, an iteration 0.4 and 0.65 per round of the
+// block's threads over its pairs of nodes; the one-iteration kernel 1.75 and
+// 8 per million nodes.  They err against the tiles (a round costs less
+// once pairs near the edge drop out): timed at 19 sizes from 61 x 31 to 512^2 in
+// FP32, exact momentum, FP16 and BF16, what they choose is never slower than one
+// iteration per launch (closest: 400^2 FP16 3.45 against 3.48 us per iteration; 256^2 1.71 |
+// 1.95 | 2.07 | 2.03 against 2.26 | 2.38 | 2.69 | 2.70), but they leave single
+// iterations at 300^2 (FP32 2.50; T = 10 takes 2.09), 333^2 and 440^2, and below
+// 100^2 a shorter T than theirs gains 3 (FP32) to 12 % (exact momentum).
 void plan_tiles(lb_ctx *ctx) {
   ctx->tile_steps = 1;
   double best = 1.75 + 8e-6 * (double)ctx->nx * ctx->ny;

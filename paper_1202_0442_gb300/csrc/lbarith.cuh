@@ -298,9 +298,11 @@ __device__ __forceinline__ void equilibrium1(const Node1<V> &n, float sc, float 
 // (keep = 1 - omega is exact): its intermediate rounding is that of (1 - omega) h,
 // none at tau = 1 and tau = 0.8, where h + omega (h_eq - h) rounds the
 // difference at the size of h; a channel started far from equilibrium
-// (f = 4 and 1) carries 3.5 times less momentum noise after 150 iterations,
-// and flows near equilibrium the same.  For omega < 1 as h + omega (h_eq - h):
-// the noise is the lower there (tau = 1.5, body force: by 1.3), and the
+// (f = 4 and 1) carries 3.5 times less momentum noise after 150 iterations;
+// flows near equilibrium (porous 256^2, 100 iterations) have the same error at
+// tau = 0.75 and 1, 1.15 times the other form's at 0.6, 1.01 at 0.52 (0.5 to 0.8 of
+// equilibrium_16's with that form).  For omega < 1 as h + omega (h_eq - h):
+// the error is the lower there (tau = 1.5: by 3), and the
 // node's sums are kept although 1 - omega may be rounded; 16-bit storage
 // always takes that form (equilibrium_16).  RX: 0 decided here, 1 the first
 // form, 2 the second (decided by the launch: both forms in one

@@ -5,8 +5,9 @@
 // before it in the stream drains: its blocks are placed once every block of
 // that kernel has exited, without waiting for the kernel's completion to
 // travel back through the front end.  Each such kernel calls dep_wait()
-// (griddepcontrol.wait) before its first global-memory access; it returns
-// once the previous kernel has completed and its writes are visible.  The
+// (griddepcontrol.wait) before its first global-memory access (k_grow_list
+// before its first access to anything the kernel in front of it writes); it
+// returns once the previous kernel has completed and its writes are visible.  The
 // order of the stream is therefore kept exactly (same results bit for bit);
 // only the launch latency between two dependent kernels is hidden.  A
 // kernel launched the ordinary way passes dep_wait() at once.
