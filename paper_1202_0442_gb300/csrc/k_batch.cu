@@ -57,7 +57,8 @@ __device__ __forceinline__ void batch_warp(const BatchLat &L, const S *fin, S *f
   if (L.pm) shift1<float, true, sizeof(S) == 2>(L.tau, n);
   else shift1<float, false, sizeof(S) == 2>(L.tau, n);
   float heq[9];
-  equilibrium1<float, false, sizeof(S) == 2>(n, 1.0f, 1.0f / 9.0f, 1.0f / 36.0f, heq);
+  if (L.pm) equilibrium1<float, true, false, sizeof(S) == 2>(n, 1.0f, 1.0f / 9.0f, 1.0f / 36.0f, heq);
+  else equilibrium1<float, false, false, sizeof(S) == 2>(n, 1.0f, 1.0f / 9.0f, 1.0f / 36.0f, heq);
   relax<sizeof(S) == 2 ? 2 : 0>(h, heq, L.omega, 1.0f - L.omega);
   if (L.sr) {
     // stochastic rounding as in the single-lattice kernels: one hash per

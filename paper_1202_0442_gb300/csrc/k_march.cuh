@@ -234,7 +234,7 @@ __device__ __forceinline__ void collide_pair(const MarchLat &p, const MarchOpen 
   n.Fy = vfma(n.rho, vset<f2>(p.ay), vset<f2>(p.fy));
   shift1<f2, PM, sizeof(S) == 2>(p.tau, n);
   f2 heq[9];
-  equilibrium1<f2, FOLD, sizeof(S) == 2>(n, p.scale, p.wa, p.wd, heq);
+  equilibrium1<f2, PM, FOLD, sizeof(S) == 2>(n, p.scale, p.wa, p.wd, heq);
   if (fields) {
     const f2 half = vset<f2>(0.5f);
     fields[0] = n.drho;

@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile(const TileArgs t) {
       nd.Fy = vfma(nd.rho, vset<f2>(p.ay), vset<f2>(p.fy));
       shift1<f2, PM, sizeof(S) == 2>(p.tau, nd);
       f2 heq[9];
-      equilibrium1<f2, FOLD, sizeof(S) == 2>(nd, p.scale, p.wa, p.wd, heq);
+      equilibrium1<f2, PM, FOLD, sizeof(S) == 2>(nd, p.scale, p.wa, p.wd, heq);
       relax<sizeof(S) == 2 ? 2 : 0>(v, heq, p.omega, p.keep);
       S a[9], b[9];
       round_pair<S, SR>(v, seed, q.selfa, q.selfb, a, b);

@@ -49,7 +49,7 @@ __device__ __forceinline__ void collide_store(const FluidArgs &p, int x, int y, 
   shift1<float, PM, sizeof(S) == 2>(p.tau[0], n);
   S *out = (S *)p.fout;
   float heq[9];
-  equilibrium1<float, FOLD, sizeof(S) == 2>(n, p.scale, p.wa[0], p.wd[0], heq);
+  equilibrium1<float, PM, FOLD, sizeof(S) == 2>(n, p.scale, p.wa[0], p.wd[0], heq);
   relax<sizeof(S) == 2 ? 2 : RX>(h, heq, p.omega[0], p.keep);
   // in stored units: FP16 is folded, the other types have no scale
   if (SR == 2) {
