@@ -881,21 +881,15 @@ bool march_ok(const lb_ctx *ctx) {
 }
 
 // The tiles of k_tile: for T iterations per launch the grid of at most one
-// block per SM whose tiles with their halo are the smallest, and the T that
-// costs the least per iteration, if that is less than the one-iteration
-// kernel's (T = 1).  Costs in us, from FP32 timings with T = 2..12: a launch
-// 1.8 and 3 per 1000 nodes read, an iteration 0.4 and 0.65 per round of the
-// block's threads over its pairs of nodes; the one-iteration kernel 1.75 and
-// 8 per million nodes.  They err against the tiles (a round costs less
-// once pairs near the edge drop out): timed at 19 sizes from 61 x 31 to 512^2 in
-// FP32, exact momentum, FP16 and BF16, what they choose is never slower than one
-// iteration per launch (closest: 400^2 FP16 3.45 against 3.48 us per iteration; 256^2 1.71 |
-// 1.95 | 2.07 | 2.03 against 2.26 | 2.38 | 2.69 | 2.70), but they leave single
-// iterations at 300^2 (FP32 2.50; T = 10 takes 2.09), 333^2 and 440^2, and below
-// 100^2 a shorter T than theirs gains 3 (FP32) to 12 % (exact momentum).
+// block per SM whose tiles with their halo are the smallest, and the cost of an
+// iteration with them, in us; tile_cost[1] is the one-iteration kernel's.  The
+// costs are fitted to FP32 timings of T = 1..12 at 17 sizes from 61 x 31 to 480^2
+// (rms 7 %): a launch 2.27 and 2.17 per 1000 nodes read, an iteration 0.26,
+// 0.89 per 512 pairs that it still advances and 0.1 per round of the block's
+// threads; the one-iteration kernel 1.80 and 7.8 per million slots.
 void plan_tiles(lb_ctx *ctx) {
   ctx->tile_steps = 1;
-  double best = 1.75 + 8e-6 * (double)ctx->nx * ctx->ny;
+  ctx->tile_cost[1] = 1.80 + 7.77e-6 * (double)ctx->g.pitch * ctx->ny;
   for (int T = 2; T <= TILE_STEPS; T++) {
     int64_t least = TILE_NODES + 1;
     for (int bx = 1; bx <= ctx->sms && bx <= ctx->nx; bx++) {
@@ -909,13 +903,42 @@ void plan_tiles(lb_ctx *ctx) {
       }
     }
     if (least > TILE_NODES) break;
+    // pairs of nodes that iterations 1..T advance: the region less n columns
+    // and rows on each side
+    const int W = ctx->tile_w[T] + 2 * T, H = (ctx->tile_h[T] + 2 * T + 1) & ~1;
+    int64_t pairs = 0;
+    for (int n = 1; n <= T; n++)
+      pairs += (int64_t)std::max(W - 2 * n, 0) * std::max((H - 1 - n) / 2 - n / 2 + 1, 0);
     const double rounds = (double)((least / 2 + TILE_THREADS - 1) / TILE_THREADS);
-    const double cost = (1.8 + 3e-3 * (double)least) / T + 0.4 + 0.65 * rounds;
-    if (cost < best) {
-      best = cost;
-      ctx->tile_steps = T;
+    ctx->tile_cost[T] = (2.27 + 2.17e-3 * (double)least + 0.894 * (double)pairs / TILE_THREADS) / T + 0.257 + 0.1 * rounds;
+    if (ctx->tile_cost[T] < ctx->tile_cost[ctx->tile_steps]) ctx->tile_steps = T;
+  }
+}
+
+// Launches for n iterations by tiles, of equal length but for one iteration,
+// their number odd or even as n is, so that the current buffer alternates as
+// documented; n where single iterations cost less.  A short call or an odd
+// rest would be cut into launches of two or three iterations, which take longer
+// than single ones on all but the smallest lattices (us per iteration, FP32:
+// 400^2 T = 2 4.62, 3 3.71, 6 2.79, single 3.08; 256^2 2.50, 2.06, 1.91 (5: 1.71), single 2.26; 64 x 32
+// 1.45, 1.14, 0.83, single 1.82).  Against single iterations, n from 3 to
+// 100, 19 sizes, FP32, exact momentum, FP16 and BF16: 0.85 in the mean, at most
+// 1.07 (1024 x 128 FP16, n = 13), where the longest launches alone were up to 1.5.
+int64_t tile_launches(const lb_ctx *ctx, int64_t n) {
+  if (ctx->tile_steps == 1 || n < 3) return n;
+  int64_t first = (n + ctx->tile_steps - 1) / ctx->tile_steps, best = n;
+  if ((first ^ n) & 1) first++;
+  double least = 0.96 * ctx->tile_cost[1] * (double)n;
+  for (int64_t l = first; l <= first + 2 && l < n; l += 2) {
+    const int64_t T = n / l, longer = n % l;
+    double cost = (double)((l - longer) * T) * ctx->tile_cost[T];
+    if (longer) cost += (double)(longer * (T + 1)) * ctx->tile_cost[T + 1];
+    if (cost < least) {
+      least = cost;
+      best = l;
     }
   }
+  return best;
 }
 
 void march_lattice(const FluidArgs &f, MarchLat &l) {
@@ -991,11 +1014,10 @@ int tile_launch(lb_ctx *ctx, int T, bool fields) {
   return LB_OK;
 }
 
-// n iterations by tiles: launches of equal length, their number odd or even
-// as n is, so that the current buffer alternates as documented
+// n iterations by tiles, if those cost less than single ones (else none)
 int tile_steps(lb_ctx *ctx, int64_t n, bool fields) {
-  int64_t launches = (n + ctx->tile_steps - 1) / ctx->tile_steps;
-  if ((launches ^ n) & 1) launches++;
+  int64_t launches = tile_launches(ctx, n);
+  if (launches == n) return LB_OK;
   while (launches > 0) {
     const int T = (int)((n + launches - 1) / launches);
     const bool last = launches == 1;
@@ -1798,7 +1820,7 @@ int lb_iteration(lb_ctx *ctx, int Nt) {
     // by twos an even number of times, so that the current buffer
     // alternates with the iterations as documented
     for (int64_t j = march ? n / 4 * 4 : 0; j > 0; j -= 2) TRY(two_steps(ctx, ctx->t + 2 == end && (thermo || out)));
-    if (several && !march && ctx->tile_steps > 1 && n > 2) TRY(tile_steps(ctx, n, thermo || out));
+    if (several && !march) TRY(tile_steps(ctx, n, thermo || out));
     while (ctx->t < end) {
       TRY(one_step(ctx, ctx->t + 1 == end && (thermo || out)));
       if (ctx->rank >= 0 && ctx->py == 1) TRY(exchange_slabs(&ctx, 1));

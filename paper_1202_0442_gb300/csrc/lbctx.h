@@ -129,6 +129,7 @@ struct lb_ctx {
   // the lattice is too large), and the number that costs the least per
   // iteration (0: not planned yet, 1: no tiles)
   int tile_w[lbk::TILE_STEPS + 1] = {0}, tile_h[lbk::TILE_STEPS + 1] = {0}, tile_steps = 0;
+  double tile_cost[lbk::TILE_STEPS + 1] = {0};  // us per iteration
   bool fields_valid = false;
   int64_t fields_step = -1;  // iteration whose end state the field planes hold
   lb_thermo_t thermo{};
