@@ -535,9 +535,9 @@ def variants(args, local, stream, flush, value_fp32):
             # two iterations per launch: half the bytes per iteration
             "roofline_frac": bpn / 2 * fluid / (ms_b * 1e-3) / 1e9 / peak,
             "state_bytes": int(2 * bpn * nodes),
-            "accuracy": ("rel. u <= 3.8e-6 on 8 sampled lattices after 5000 iterations (exact momentum pairs): meets 1e-5"
+            "accuracy": ("rel. u <= 2.5e-6 on 8 sampled lattices after 5000 iterations (exact momentum pairs): meets 1e-5"
                          if st == "fp32" else
-                         "rel. u up to 1.4e-2 on 8 sampled lattices after 5000 iterations: "
+                         "rel. u up to 1.2e-2 on 8 sampled lattices after 5000 iterations: "
                          "misses 2e-3 on the slow ones")}
         del b, lats
     out["batched_fp16"]["speedup_vs_fp32_batched"] = (out["batched"]["ms_per_iteration_batched"]
